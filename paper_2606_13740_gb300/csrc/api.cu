@@ -101,9 +101,11 @@ Layout make_layout(const dllm_config& c) {
     L.off_x0 = take(T * 4);
     L.off_conf = take(T * 4);
     L.off_tokconf = take(T * 4);
-    // chained projections: per phase slot, split partials (one per CTA), tile tickets (one per
-    // 128-byte line) and tile completion flags
-    L.part_floats = static_cast<size_t>(kMaxSMs) * 256 * 128;
+    // chained projections: per phase slot, split partials (two per CTA, one in 32-token tiles; a
+    // token tile is never wider than the tokens), tile tickets (one per 128-byte line) and tile
+    // completion flags
+    const int nt_max = std::min(256, rup(L.max_tok, 32));
+    L.part_floats = static_cast<size_t>(kMaxSMs) * (nt_max > 32 ? 2 : 1) * nt_max * 128;
     L.off_part = take(L.part_floats * 4 * kMaxPhases);
     const int mt_max = std::max(std::max(L.head_tiles, L.gu_rows / 128), std::max(L.qkv_rows, L.d_rows) / 128);
     L.done_len = mt_max * ((L.max_tok + 255) / 256 + 1);

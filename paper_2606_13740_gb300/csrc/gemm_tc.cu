@@ -20,13 +20,17 @@
 // that read the same weight tile for different token tiles run about in step
 // and share it through L2) is cut into one contiguous range per CTA, so
 // every SM streams the same number of weight bytes whatever the tile count.
-// A tile cut between CTAs is finished by the CTA holding its first k-blocks,
-// which are the end of that CTA's range: the other parts store fp32 partials
-// and publish each on its own flag, and the finishing CTA polls every part's
-// flag at once (bounded), bulk-copies each part's slice into shared memory as
-// soon as it is published and adds them to its own accumulator in part order
-// (deterministic).  Every CTA waits only on CTAs that wait on nothing later
-// than it, and the grid never exceeds the SM count, so all are resident.
+// A tile cut between CTAs (its parts, in k order) is finished from fp32
+// partials in L2, each part published on a flag of its own, summed in part
+// order (deterministic).  A 32-token tile is finished by the CTA holding its
+// first k-blocks, which are the end of that CTA's range.  A wider tile is
+// finished 32 columns at a time by every CTA whose range ends in it, all of
+// the tile's parts but the last: one finisher took the columns one after
+// another, and with five parts and 256 tokens (the output projection of a
+// 251-token window) that was 40 slices in a row on a sixth of the SMs (a layer
+// at 251 tokens 190 -> 132 us, at 160 tokens and ffn 18944 163 -> 104 us).  Every CTA waits only on CTAs
+// that wait on nothing later than it, and the grid never exceeds the SM count,
+// so all are resident.
 // The weights (the context's, stored tile-major) arrive as one contiguous
 // bulk copy per 16 KB tile; row-major weights of the single-projection entry
 // points arrive through a 2-D tensor map.
@@ -50,7 +54,10 @@ constexpr int kBK = 64;     // K elements per stage: one 128-byte swizzle row
 constexpr uint32_t kABytes = kBM * kBK * 2;
 constexpr int kFullSmem = 227 * 1024;
 static int g_stream_budget = kChainSmemShared;  // single projections: shared-memory plan
-constexpr int kTicketStride = 32;  // a tile's part flags: one 128-byte line (parts 1..31)
+constexpr int kTicketStride = 32;  // a tile's part flags: one 128-byte line (parts 0..30) ...
+constexpr int kStgBytes = 32 * kBM * 2;  // the epilogue's staging of a 32-token chunk's bf16 outputs
+constexpr int kTailFloats = 256 + 1024 + 256 + 128 + 256;  // EpiSmem's arrays
+constexpr int kOwnerCount = 31;    // ... and the count of its owners that are done
 constexpr int kEpiGroup = 16;      // epilogue columns processed side by side: half a 32-token chunk
 constexpr int kEpiWarps = 8;       // two per TMEM lane quarter, one per half chunk
 constexpr int kEpiThreads = kEpiWarps * 32;
@@ -78,8 +85,8 @@ struct EpiSmem {
     float* red;   // [4][256] cross-warp / quarter partial sums
     int* kvs;     // [256] per-sequence first window position (QKV); current ids of the token tile (LM head)
     float* theta; // [128] rotation frequency of each tile row's feature pair (QKV)
-    uint8_t* stg;  // staging of a 32-token chunk's bf16 outputs, 8 KB (for tiles of more than one chunk its
-                   // own memory: the next chunk's partial slices arrive meanwhile)
+    float* step;  // [128][2] its rotation from one position to the next (cos, sin)
+    uint8_t* stg;  // staging of a 32-token chunk's bf16 outputs (kStgBytes; wide tiles: two of them in turn)
     const int* rows;  // the launch's device-resolved row count (-1: the plans as given)
 };
 
@@ -171,6 +178,7 @@ struct QkvPlan {
 };
 __device__ __forceinline__ QkvPlan qkv_plan(const EpiArgs& ep, const GemmPlan& p, int mt, int col0, int rt,
                                             const EpiSmem& sm, int e, int half) {
+    const int hd_sh = ep.hd == 128 ? 7 : 6, hd_m = ep.hd - 1;  // the head dim is 64 or 128
     QkvPlan q;
     const int row = mt * kBM + rt;
     // q rows [0, qd), k rows [qd, qd + kvd), v rows [qd + kvd, qd + 2 kvd): the same part for
@@ -178,36 +186,35 @@ __device__ __forceinline__ QkvPlan qkv_plan(const EpiArgs& ep, const GemmPlan& p
     const int qd = ep.H * ep.hd;
     q.part = row < qd ? 0 : (row < ep.v_row0 ? 1 : 2);
     const int f = row - (q.part == 0 ? 0 : (q.part == 1 ? qd : ep.v_row0));
-    q.pp = f % ep.hd;
+    q.pp = f & hd_m;
     q.fi = (q.pp >> 1) + (q.pp & 1) * (ep.hd >> 1);
     q.theta = sm.theta[rt];
-    q.bl = col0 / ep.T;
-    q.run = min(col0 + 31, p.N - 1) / ep.T == q.bl && min(col0 + 31, p.N - 1) - q.bl * ep.T < ep.Tw;
+    q.bl = ep.n_seq > 1 ? col0 / ep.T : 0;
+    q.run = (ep.n_seq == 1 || min(col0 + 31, p.N - 1) / ep.T == q.bl) && min(col0 + 31, p.N - 1) - q.bl * ep.T < ep.Tw;
     q.cn = 1.0f;
     q.sn = 0.0f;
     q.cd = 1.0f;
     q.sd = 0.0f;
     if (q.part < 2 && q.run) {
         const float2 a = rot_cs(static_cast<float>(sm.kvs[q.bl] + (col0 + kEpiGroup * half - q.bl * ep.T)) * q.theta);
-        const float2 d = rot_cs(q.theta);
         q.cn = a.x;
         q.sn = a.y;
-        q.cd = d.x;
-        q.sd = d.y;
+        q.cd = sm.step[2 * rt];
+        q.sd = sm.step[2 * rt + 1];
     }
     const int tok = e >> 3, f0 = (e & 7) * 16;
     const int col = col0 + tok;
     q.dst = nullptr;
     q.bad = false;
     if (col < p.N) {
-        const int b = min(col / ep.T, ep.n_seq - 1);
+        const int b = ep.n_seq > 1 ? min(col / ep.T, ep.n_seq - 1) : 0;
         const int ts = col - b * ep.T;
         const bool tracked = ts >= ep.Tw;  // sparse cache refresh: K/V to the side buffers
         const int pos = tracked ? ep.trk[b * ep.R + ts - ep.Tw] : sm.kvs[b] + ts;
         const int base = q.part == 0 ? 0 : (q.part == 1 ? qd : ep.v_row0);  // the part's first row
-        const int head = (mt * kBM - base + f0) / ep.hd;
+        const int head = (mt * kBM - base + f0) >> hd_sh;
         const int heads = q.part == 0 ? ep.H : ep.Hkv;  // q: query heads; K/V: the cache's heads
-        const int fi0 = f0 % ep.hd;
+        const int fi0 = f0 & hd_m;
         if (tracked && q.part > 0) {
             if (pos >= 0) {
                 __nv_bfloat16* side = q.part == 1 ? ep.kside : ep.vside;
@@ -235,12 +242,14 @@ __device__ __forceinline__ QkvPlan qkv_plan(const EpiArgs& ep, const GemmPlan& p
 // Residual epilogue in two passes (PASS 1: the bf16 copy, the next projection's operand, and
 // the RMSNorm partial sums; PASS 2: the fp32 residual and the sums' store), so the tile can be
 // published to the next phase's operand producer between them; PASS 0: both at once.
-template <int EPI, int PASS = 0>
+// ALT: the caller alternates between two staging buffers, so that the barrier between a chunk's
+// staging and its stores also covers the buffer's next use.
+template <int EPI, int PASS = 0, bool ALT = false>
 __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& p, int mt, int col0, int c_in,
                                              int rt, uint32_t t_src, uint32_t t_x, const EpiSmem& sm,
                                              int e, int half, int quarter, int lane, int* status,
                                              const float* a_in = nullptr, const QkvPlan* qkv_pre = nullptr,
-                                             const float* x_in = nullptr) {
+                                             bool x_added = false, int buf = 0) {
     // col0: the chunk's first token column; c_in: its offset inside the token tile (index into
     // the tile's RMSNorm scales and staged ids).  The thread's 16 accumulator columns come from
     // a_in (a finisher's sum of the parts, in registers), else from TMEM at t_src.  The old
@@ -250,6 +259,7 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
     // chunk.  qkv_pre: the QKV plan, built ahead (null: built here).
     constexpr int GW = kEpiGroup;  // columns per group
     constexpr int LS = 32 / GW;    // lanes sharing one column's sum after the scatter
+    uint8_t* const stg = ALT ? sm.stg + buf * kStgBytes : sm.stg;
     const int row = mt * kBM + rt;
     const bool scale = (EPI == EPI_QKV || EPI == EPI_SWIGLU || EPI == EPI_LMHEAD) && ep.sq_in != nullptr;
     QkvPlan qp;
@@ -300,9 +310,9 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
             } else {
                 if (t_x) {
                     tmem_ld_32xn<GW>(t_x + static_cast<uint32_t>(GW * g), xo);
-                } else if (x_in) {
+                } else if (x_added) {
 #pragma unroll
-                    for (int u = 0; u < GW; ++u) xo[u] = x_in[u];
+                    for (int u = 0; u < GW; ++u) xo[u] = 0.0f;
                 } else {
 #pragma unroll
                     for (int u = 0; u < GW; ++u)
@@ -324,7 +334,7 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
                         ep.xb[o] = __float2bfloat16_rn(xo[u]);
                     }
                 } else if constexpr (PASS == 1) {  // token-major staging, stored below in 16-byte pieces
-                    reinterpret_cast<__nv_bfloat16*>(sm.stg)[(GW * g + u) * kBM + rt] = __float2bfloat16_rn(xo[u]);
+                    reinterpret_cast<__nv_bfloat16*>(stg)[(GW * g + u) * kBM + rt] = __float2bfloat16_rn(xo[u]);
                 } else {  // fp32: a warp's 32 rows of one token are one 128-byte line
                     if (ok) ep.out[static_cast<size_t>(cg + u) * ep.ld_out + row] = xo[u];
                 }
@@ -367,7 +377,7 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
             for (int u = 0; u < GW; ++u) xp[u] = __shfl_xor_sync(0xffffffffu, a[u], 1);
             // staged token-major in feature order ([32][128]: the tile's head(s) side by side),
             // stored below in 16-byte pieces
-            __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(sm.stg) + (rt / ep.hd) * ep.hd + fi;
+            __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(stg) + (rt / ep.hd) * ep.hd + fi;
 #pragma unroll
             for (int u = 0; u < GW; ++u) {
                 float x = a[u];
@@ -382,7 +392,7 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
 #pragma unroll
             for (int u = 0; u < GW; ++u) up[u] = __shfl_xor_sync(0xffffffffu, a[u], 1);
             // staged token-major ([32][64] features), stored below in 16-byte pieces
-            __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(sm.stg) + (rt >> 1);
+            __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(stg) + (rt >> 1);
 #pragma unroll
             for (int u = 0; u < GW; ++u) {
                 const __nv_bfloat16 hv = __float2bfloat16_rn(__fdividef(a[u], 1.0f + __expf(-a[u])) * up[u]);
@@ -433,12 +443,12 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
         if (qp.dst) {
             const int t = e, tok = t >> 3, f0 = (t & 7) * 16;
             const uint4* src =
-                reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(sm.stg) + tok * kBM + f0);
+                reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(stg) + tok * kBM + f0);
 #pragma unroll
             for (int i = 0; i < 2; ++i) qp.dst[i] = src[i];
         }
         if (qp.bad) atomicOr(status, kStatusBadIndex);
-        named_bar(1, kEpiThreads);  // the staging memory is free again
+        if (!ALT) named_bar(1, kEpiThreads);  // the staging memory is free again
     } else if constexpr (EPI == EPI_SWIGLU) {
         // thread t stores token t/8, features 8 (t%8) .. +7 of the tile's 64
         named_bar(1, kEpiThreads);
@@ -446,11 +456,11 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
         const int col = col0 + tok;
         if (col < p.N) {
             const uint4* src =
-                reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(sm.stg) + tok * 64 + f0);
+                reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(stg) + tok * 64 + f0);
             const int fg = mt * 64 + f0;  // F is a multiple of 8: each 8-feature piece is all in or all out
             if (fg < ep.F) *reinterpret_cast<uint4*>(ep.h + static_cast<size_t>(col) * ep.F + fg) = *src;
         }
-        named_bar(1, kEpiThreads);
+        if (!ALT) named_bar(1, kEpiThreads);
     }
     if constexpr (EPI == EPI_RESID && PASS == 1) {
         // the staged chunk: thread t stores token t/8, features 16 (t%8) .. +15 of the tile
@@ -459,12 +469,12 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
         const int col = col0 + tok;
         if (col < p.N) {
             const uint4* src =
-                reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(sm.stg) + tok * kBM + f0);
+                reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(stg) + tok * kBM + f0);
             uint4* dst = reinterpret_cast<uint4*>(ep.xb + static_cast<size_t>(col) * ep.ld_out + mt * kBM + f0);
 #pragma unroll
             for (int i = 0; i < 2; ++i) dst[i] = src[i];
         }
-        named_bar(1, kEpiThreads);  // the staging memory is free again
+        if (!ALT) named_bar(1, kEpiThreads);  // the staging memory is free again
     }
     if constexpr (EPI == EPI_RESID && PASS == 0) {
         named_bar(1, kEpiThreads);
@@ -540,7 +550,7 @@ constexpr int kMaxDepTiles = 1024;  // the operand producer keeps a readiness bi
 struct ChainEpiState {
     int acc;
     uint32_t acc_phase;
-    uint32_t red_phase;
+    int buf;  // wide tiles: the staging buffer of the next chunk
 };
 
 __device__ __forceinline__ int chain_tag(const ChainArgs& ca) {
@@ -588,13 +598,20 @@ __device__ __forceinline__ bool wait_parts(const int* flags, int q0, int qn, int
     return !named_bar_any(1, kEpiThreads, *s_abort != 0);
 }
 
+// The partial slot of part `part` (of its tile) of CTA `cta`: a CTA whose range both ends one
+// split tile and begins another may store a partial of each (p.slots == 2).
+template <bool WIDE>
+__device__ __forceinline__ size_t part_slot(const GemmPlan& p, int cta, int part) {
+    if (!WIDE) return static_cast<size_t>(cta);
+    return static_cast<size_t>(cta) * p.slots + (p.slots == 2 && part == 0 ? 1 : 0);
+}
+
 // The epilogue warps' share of one phase: every tile of this CTA's range.
 // WIDE: token tiles of several 32-token chunks (split tiles reduced through the staging
 // slots); else one chunk (split tiles reduced in registers): each its own code.
 template <int EPI, int DP, bool WIDE>
-__device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph, int tag, uint8_t* red_stage,
-                                                  uint64_t* tfull, uint64_t* tempty, uint64_t* redbar,
-                                                  volatile int* s_abort, uint32_t tmem_base, const EpiSmem& esm,
+__device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph, int tag, uint64_t* tfull, uint64_t* tempty,
+                                                     volatile int* s_abort, uint32_t tmem_base, const EpiSmem& esm,
                                                   ChainEpiState& es) {
     const ChainPhase& P = ca.ph[ph];
     const GemmPlan p = phase_plan(P, *esm.rows);
@@ -606,10 +623,9 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
     const int half = ew >> 2;                         // columns 16 half .. +15 of every chunk
     const int quarter = warp & 3;                     // TMEM lane quarter = tile rows 32 quarter ..
     const int rt = quarter * 32 + lane;
-    const int G = p.grid;
-    if (static_cast<int>(blockIdx.x) >= G) return;
-    const long long it0 = range_begin(blockIdx.x, p.total, G);
-    const long long it1 = range_begin(blockIdx.x + 1, p.total, G);
+    if (static_cast<int>(blockIdx.x) >= p.grid) return;
+    const int it0 = static_cast<int>(range_begin(blockIdx.x, p.total, p.grid));
+    const int it1 = static_cast<int>(range_begin(blockIdx.x + 1, p.total, p.grid));
     if (it0 >= it1) return;
     unsigned long long* tr = ep.trace ? ep.trace + static_cast<size_t>(blockIdx.x) * kTrSlots : nullptr;
     if (tr && threadIdx.x == 64) {
@@ -630,7 +646,13 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
     if (tr && threadIdx.x == 64) tr[kTrDepWait] = global_ns();
     if constexpr (EPI == EPI_QKV) {
         for (int b = e; b < ep.n_seq; b += kEpiThreads) esm.kvs[b] = ep.seq_kv[b];
-        if (half == 0) esm.theta[rt] = ep.theta[(rt % ep.hd) >> 1];
+        if (half == 0) {
+            const float th = ep.theta[(rt % ep.hd) >> 1];
+            const float2 d = rot_cs(th);
+            esm.theta[rt] = th;
+            esm.step[2 * rt] = d.x;
+            esm.step[2 * rt + 1] = d.y;
+        }
         named_bar(1, kEpiThreads);
     }
     const int nchunks = p.ntile / 32;
@@ -639,20 +661,20 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
     // TMEM: two accumulators of acc_cols columns, then (token tiles up to 128) the staged old
     // residual of the finisher's tile, x_cols columns
     const uint32_t t_x =
-        ca.x_cols ? tmem_base + static_cast<uint32_t>(2 * ca.acc_cols) + (static_cast<uint32_t>(quarter * 32) << 16)
+        !WIDE && ca.x_cols ? tmem_base + static_cast<uint32_t>(2 * ca.acc_cols) + (static_cast<uint32_t>(quarter * 32) << 16)
                   : 0u;
     int rs_nt = -1, ids_nt = -1;
-    long long prepared = -1;
+    int prepared = -1;
     float v[16];
     // Work a finisher needs before its accumulator: the RMSNorm scale of its token tile, the
     // LM head's current ids of the token tile, and (residual, 32-token tiles) the old x staged
     // in TMEM.  Done as early as possible: for a contributor tile, ahead of it for the finisher
     // tile that follows in the range.
-    auto prepare = [&](long long ptile) {
+    auto prepare = [&](int ptile) {
         if (ptile == prepared) return;
         prepared = ptile;
-        const int pnt = static_cast<int>(ptile / p.m_tiles);
-        const int pmt = static_cast<int>(ptile - static_cast<long long>(pnt) * p.m_tiles);
+        const int pnt = ptile / p.m_tiles;
+        const int pmt = ptile - pnt * p.m_tiles;
         if constexpr (EPI == EPI_QKV || EPI == EPI_SWIGLU || EPI == EPI_LMHEAD) {
             if (ep.sq_in && pnt != rs_nt) {
                 compute_norm_scale(ep, p, pnt, esm, e);
@@ -683,22 +705,42 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
             }
         }
     };
-    for (long long it = it0; it < it1;) {
-        const long long tile = it / p.kb;
-        const int k_lo = static_cast<int>(it - tile * p.kb);
-        const long long tend = (tile + 1) * p.kb;
-        const int k_hi = static_cast<int>((it1 < tend ? it1 : tend) - tile * p.kb);
-        const int nt = static_cast<int>(tile / p.m_tiles);
-        const int mt = static_cast<int>(tile - static_cast<long long>(nt) * p.m_tiles);
-        const bool whole = (k_lo == 0 && k_hi == p.kb);
-        int c_first = 0, c_last = 0;
-        bool reducer = false;
-        if (!whole) {
-            c_first = owner_of(tile * p.kb, p.total, G);
-            c_last = owner_of(tile * p.kb + p.kb - 1, p.total, G);
-            reducer = static_cast<int>(blockIdx.x) == c_first;
+    // Wide tiles read the old residual from global memory (TMEM has no room to stage it; a warp's
+    // 32 rows of one token are one 128-byte line), the first chunk's before the accumulator is
+    // ready and each further one's behind the chunk before it.  L2 only: other CTAs wrote them.
+    float xw[kEpiGroup];
+    auto load_x = [&](int xmt, int xnt, int c) {
+        const int xrow = xmt * kBM + rt;
+#pragma unroll
+        for (int u = 0; u < kEpiGroup; ++u) {
+            const int xcol = xnt * p.ntile + c * 32 + half * kEpiGroup + u;
+            xw[u] = (xrow < p.M && xcol < p.N) ? __ldcg(ep.out + static_cast<size_t>(xcol) * ep.ld_out + xrow) : 0.0f;
         }
+    };
+    for (int it = it0; it < it1;) {
+        const int tile = it / p.kb;
+        const int k_lo = it - tile * p.kb;
+        const int tend = (tile + 1) * p.kb;
+        const int k_hi = min(it1, tend) - tile * p.kb;
+        const int nt = tile / p.m_tiles;
+        const int mt = tile - nt * p.m_tiles;
+        const bool whole = (k_lo == 0 && k_hi == p.kb);
+        // A split tile's parts are CTAs c_first .. c_last, in k order.  Its columns are finished
+        // by n_own of them: one-chunk tiles (and callers with one partial slot a CTA) by the
+        // first part; wider ones chunk by chunk by every part but the last, whose CTA goes on
+        // to a tile of its own.  Every owner's part is the end of its CTA's range, so a CTA
+        // finishes columns of one tile at most.
+        int c_first = 0, c_last = 0, n_own = 0;
+        if (!whole) {
+            c_first = owner_of(tile * p.kb, p.total, p.grid);
+            c_last = owner_of(tile * p.kb + p.kb - 1, p.total, p.grid);
+            n_own = WIDE && p.slots == 2 ? min(nchunks, max(1, c_last - c_first)) : 1;
+        }
+        const int part = static_cast<int>(blockIdx.x) - c_first;
+        const bool reducer = !whole && part < n_own;
         const bool finisher = whole || reducer;
+        if constexpr (WIDE && EPI == EPI_RESID)
+            if (finisher) load_x(mt, nt, whole ? 0 : part);
         // a contributor's range goes on into a tile whose first k-blocks it holds: a finisher
         if (finisher) prepare(tile);
         else if (tend < it1) prepare(tile + 1);
@@ -707,10 +749,7 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
         const bool late_acc = reducer && !WIDE;
         if (!late_acc) {
             mbar_wait(&tfull[es.acc], es.acc_phase, s_abort, status);
-            if (named_bar_any(1, kEpiThreads, *s_abort != 0)) {
-                cp_async_wait<0>();  // no copy lands in shared memory after the launch has ended
-                return;
-            }
+            if (named_bar_any(1, kEpiThreads, *s_abort != 0)) return;
             if (tr && threadIdx.x == 64) {
                 tr[kTrAccReady] = global_ns();
                 tr[kTrTile] = static_cast<unsigned long long>(tile);
@@ -721,144 +760,160 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
                                (static_cast<uint32_t>(quarter * 32) << 16);
         if (whole) {
             // the compact epilogue per 32-column chunk, straight from the accumulator in TMEM
+#pragma unroll 1
             for (int c = 0; c < nchunks; ++c) {
-                epilogue_c32<EPI, kPass1>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
-                                          t_acc + static_cast<uint32_t>(c * 32),
-                                          t_x ? t_x + static_cast<uint32_t>(c * 32) : 0u, esm, e, half, quarter, lane,
-                                          status);
-            }
-        } else if (!reducer) {
-            float* my_part = P.partials + static_cast<size_t>(blockIdx.x) * slot_floats;
-            for (int c = 0; c < nchunks; ++c) {
-                tmem_ld_32x16(t_acc + static_cast<uint32_t>(c * 32 + half * 16), v);
-                float4* dst = reinterpret_cast<float4*>(my_part);
+                constexpr bool x_ahead = WIDE && EPI == EPI_RESID;
+                if constexpr (x_ahead) {
+                    tmem_ld_32x16(t_acc + static_cast<uint32_t>(c * 32 + half * 16), v);
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    dst[static_cast<size_t>(c * 8 + half * 4 + j) * kBM + rt] =
-                        make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    for (int j = 0; j < 16; ++j) v[j] += xw[j];
+                    if (c + 1 < nchunks) load_x(mt, nt, c + 1);
+                }
+                epilogue_c32<EPI, kPass1, WIDE>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
+                                                t_acc + static_cast<uint32_t>(c * 32),
+                                                t_x ? t_x + static_cast<uint32_t>(c * 32) : 0u, esm, e, half, quarter,
+                                                lane, status, x_ahead ? v : nullptr, nullptr, x_ahead, es.buf);
+                es.buf ^= 1;
             }
-            // the partial is in registers' way out: the accumulator is free again
-            tc_fence_before();
-            mbar_arrive(&tempty[es.acc]);
+        }
+        int* const flags = P.tickets + static_cast<size_t>(tile) * kTicketStride;
+        if (!whole && (WIDE ? (!reducer || n_own > 1) : !reducer)) {
+            // the chunks that other parts finish, for them
+            float* my_part = P.partials + part_slot<WIDE>(p, blockIdx.x, part) * slot_floats;
+#pragma unroll 1
+            for (int c = WIDE ? half : 0; c < nchunks; c += WIDE ? 2 : 1) {
+                if (WIDE && reducer && c % n_own == part) continue;
+                float4* dst = reinterpret_cast<float4*>(my_part) + static_cast<size_t>(c * 8) * kBM + rt;
+                if constexpr (WIDE) {  // a warp takes every other chunk whole: one TMEM wait per 32 columns
+                    float w[32];
+                    tmem_ld_32x32(t_acc + static_cast<uint32_t>(c * 32), w);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        dst[static_cast<size_t>(j) * kBM] = make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+                } else {
+                    tmem_ld_32x16(t_acc + static_cast<uint32_t>(half * 16), v);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        dst[static_cast<size_t>(half * 4 + j) * kBM] =
+                            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                }
+            }
+            if (!reducer) {  // the accumulator is free again
+                tc_fence_before();
+                mbar_arrive(&tempty[es.acc]);
+            }
             named_bar(1, kEpiThreads);
             if (threadIdx.x == 64) {  // part q of the tile publishes its partial on flag q
                 if (tr) tr[kTrPartStored] = global_ns();
-                st_release(&P.tickets[tile * kTicketStride + (static_cast<int>(blockIdx.x) - c_first)], tag);
+                st_release(flags + part, tag);
             }
         }
         if (reducer) {
             // Part q's partial, chunk c (32 columns), is the contiguous 16 KB slice [c*8 + j][row]
-            // float4.  The slices go through the nsl staging slots (one or two) in one stream,
-            // chunk-major (slice s = chunk s / (nparts-1), part s % (nparts-1) + 1, slot s % nsl):
-            // each copy is issued as soon as its part has published (flag q == tag) and its
-            // slot's previous slice is added, so a chunk's slices arrive during the previous
-            // chunk's epilogue.  The sum runs over q in order, so it does not depend on the arrival
-            // order.  (Tiles of one 32-token chunk take the direct path below instead.)
+            // float4.  A thread loads its 16 columns of its row of every part straight into
+            // registers, up to DP parts at a time once their flags are seen, so the parts cost a
+            // round trip to L2 per group.  The sum runs over the parts in order, so it does not
+            // depend on the arrival order.
             const int nparts = c_last - c_first + 1;
-            const int np1 = nparts - 1;
-            const int nslices = nchunks * np1;
-            int* flags = &P.tickets[tile * kTicketStride];
-            constexpr uint32_t slice_bytes = 32 * kBM * 4;
-            const int nsl = ca.red_bytes >= 2 * static_cast<int>(slice_bytes) ? 2 : 1;
-            uint32_t ready = 0;     // warp 2: parts seen published (bit q)
-            uint32_t inflight = 0;  // thread 64: slots with a copy not yet waited for
-            // warp 2, warp-uniform: make sure slice s's part has published, polling every part's
-            // flag at once (lane i reads flag i, so one round trip covers them all), then thread
-            // 64 issues the copy
-            auto issue = [&](int si) {
-                const int c = si / np1, q = si - c * np1 + 1;
-                if (c == 0) {
-                    const long long t0 = spin_clock();
-                    while (!(ready >> q & 1u)) {
-                        const bool ok = lane >= 1 && lane < nparts && ld_acquire(flags + lane) == tag;
-                        ready |= __ballot_sync(0xffffffffu, ok);
-                        if (ready >> q & 1u) break;
-                        int give_up = 0;
-                        if (lane == 0) give_up = (*s_abort || spin_clock() - t0 > kWaitLimitCycles) ? 1 : 0;
-                        if (__shfl_sync(0xffffffffu, give_up, 0)) {  // warp-uniform decision
-                            if (lane == 0 && !*s_abort) {
-                                *s_abort = 1;
-                                atomicOr(status, kStatusTimeout);
-                            }
-                            return;
-                        }
-                        __nanosleep(32);
-                    }
-                }
-                if (lane == 0) {
-                    fence_proxy_async_global();
-                    fence_proxy_async_smem();  // the slot was last touched by generic accesses
-                    const int sl = si & (nsl - 1);
-                    mbar_arrive_expect_tx(redbar + sl, slice_bytes);
-                    bulk_load(red_stage + static_cast<size_t>(sl) * slice_bytes,
-                              P.partials + static_cast<size_t>(c_first + q) * slot_floats +
-                                  static_cast<size_t>(c) * 32 * kBM,
-                              slice_bytes, redbar + sl);
-                    inflight |= 1u << sl;
+            // The tile's parts but this one, i = 0 .. nparts-2: DP of them, from i0 on, of chunk c
+            // into registers.  L2 only (.cg): other CTAs wrote these lines, and the next launch
+            // writes the same slots again.  A group's loads go out without a branch (the index
+            // held at the last part); its adds stop at the last part.
+            float4 a[DP][4];
+            auto load_group = [&](int c, int i0) {
+#pragma unroll
+                for (int g = 0; g < DP; ++g) {
+                    const int i = min(i0 + g, nparts - 2), q = i + (i >= part ? 1 : 0);
+                    const float4* src = reinterpret_cast<const float4*>(
+                        P.partials + part_slot<WIDE>(p, c_first + q, q) * slot_floats);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        a[g][j] = (!WIDE || g == 0 || i0 + g < nparts - 1)
+                                      ? __ldcg(src + static_cast<size_t>(c * 8 + half * 4 + j) * kBM + rt)
+                                      : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 }
             };
-            // A 32-token tile (one chunk) skips the staging: each thread's 16 columns of its row of
-            // every part come straight into registers, up to DP parts at a time once
-            // their flags are seen, so the parts cost one round trip to L2 instead of a copy each
-            // (the same sum, in the same order, bit for bit).
-            constexpr bool direct = !WIDE;
             if (tr && threadIdx.x == 64) tr[kTrPartStored] = global_ns();
-            // the QKV plan of a one-chunk tile does not need the sum: built while the parts arrive
-            QkvPlan qpre;
-            if constexpr (EPI == EPI_QKV) {
-                if (direct) qpre = qkv_plan(ep, p, mt, nt * p.ntile, rt, esm, e, half);
-            }
-            if (ew == 0 && !direct) {
-                if (nslices > 0) issue(0);
-                if (nslices > 1 && nsl > 1) issue(1);
-            }
-            bool stop = false;
-            int si = 0;
-            for (int c = 0; c < nchunks && !stop; ++c) {
-                if (direct) {
-                    // The last part holds the tile's last k-blocks at the start of its CTA's range:
-                    // it is fetched before the own accumulator is waited for (it usually finished
-                    // earlier, and then costs nothing) and added after the middle parts, which
-                    // follow in groups (the sum in part order).
-                    if (!wait_parts(flags, nparts - 1, 1, tag, ew, lane, s_abort, status)) {
-                        stop = true;
-                        break;
-                    }
-                    const float4* srcl = reinterpret_cast<const float4*>(P.partials + static_cast<size_t>(c_last) * slot_floats);
-                    float4 al[4];
+            if constexpr (!WIDE) {
+                // the QKV plan of a one-chunk tile does not need the sum: built while the parts arrive
+                QkvPlan qpre;
+                if constexpr (EPI == EPI_QKV) qpre = qkv_plan(ep, p, mt, nt * p.ntile, rt, esm, e, half);
+                // The last part holds the tile's last k-blocks at the start of its CTA's range:
+                // it is fetched before the own accumulator is waited for (it usually finished
+                // earlier, and then costs nothing) and added after the middle parts, which
+                // follow in groups (the sum in part order).
+                if (!wait_parts(flags, nparts - 1, 1, tag, ew, lane, s_abort, status)) return;
+                const float4* srcl =
+                    reinterpret_cast<const float4*>(P.partials + static_cast<size_t>(c_last) * slot_floats);
+                float4 al[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) al[j] = __ldcg(srcl + static_cast<size_t>(half * 4 + j) * kBM + rt);
-                    mbar_wait(&tfull[es.acc], es.acc_phase, s_abort, status);
-                    if (named_bar_any(1, kEpiThreads, *s_abort != 0)) {
-                        stop = true;
-                        break;
-                    }
-                    if (tr && threadIdx.x == 64) {
-                        tr[kTrAccReady] = global_ns();
-                        tr[kTrTile] = static_cast<unsigned long long>(tile);
-                    }
-                    tc_fence_after();
-                    tmem_ld_32x16(t_acc + static_cast<uint32_t>(half * 16), v);  // own (first) k-range
-                    for (int q0 = 1; q0 < nparts - 1; q0 += DP) {
-                        const int qn = min(DP, nparts - 1 - q0);
-                        if (!wait_parts(flags, q0, qn, tag, ew, lane, s_abort, status)) {
-                            stop = true;
-                            break;
+                for (int j = 0; j < 4; ++j) al[j] = __ldcg(srcl + static_cast<size_t>(half * 4 + j) * kBM + rt);
+                mbar_wait(&tfull[es.acc], es.acc_phase, s_abort, status);
+                if (named_bar_any(1, kEpiThreads, *s_abort != 0)) return;
+                if (tr && threadIdx.x == 64) {
+                    tr[kTrAccReady] = global_ns();
+                    tr[kTrTile] = static_cast<unsigned long long>(tile);
+                }
+                tc_fence_after();
+                tmem_ld_32x16(t_acc + static_cast<uint32_t>(half * 16), v);  // own (first) k-range
+                for (int q0 = 1; q0 < nparts - 1; q0 += DP) {
+                    const int qn = min(DP, nparts - 1 - q0);
+                    if (!wait_parts(flags, q0, qn, tag, ew, lane, s_abort, status)) return;
+                    load_group(0, q0 - 1);
+#pragma unroll
+                    for (int g = 0; g < DP; ++g)
+                        if (g < qn) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                v[4 * j] += a[g][j].x;
+                                v[4 * j + 1] += a[g][j].y;
+                                v[4 * j + 2] += a[g][j].z;
+                                v[4 * j + 3] += a[g][j].w;
+                            }
                         }
-                        // L2 only (.cg): other CTAs wrote these lines, and the next launch writes
-                        // the same slots again.  A group's loads go out unconditionally (the slot
-                        // index held at the last part), its adds stop at the group's last part.
-                        float4 a[DP][4];
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    v[4 * j] += al[j].x;
+                    v[4 * j + 1] += al[j].y;
+                    v[4 * j + 2] += al[j].z;
+                    v[4 * j + 3] += al[j].w;
+                }
+                if (threadIdx.x == 64) {
+                    for (int q = 1; q < nparts; ++q) flags[q] = 0;  // ready for the next launch
+                    if (tr) {
+                        tr[kTrTicket] = global_ns();
+                        tr[kTrReduced] = global_ns();
+                        tr[kTrIsLast] = 1;
+                    }
+                }
+                // the compact epilogue on the sum in registers (the residual's first pass
+                // leaves the new residual in the still owned accumulator, for the second)
+                epilogue_c32<EPI, kPass1>(ep, p, mt, nt * p.ntile, 0, rt, t_acc, t_x, esm, e, half, quarter, lane,
+                                          status, v, EPI == EPI_QKV ? &qpre : nullptr);
+            } else {
+                // every part's flag at once (a sole owner's own part is its accumulator)
+                const int q_from = n_own > 1 ? 0 : 1;
+                if (!wait_parts(flags, q_from, nparts - q_from, tag, ew, lane, s_abort, status)) return;
+                if (tr && threadIdx.x == 64) tr[kTrTicket] = global_ns();
+                // a chunk's first group of parts is loaded a chunk ahead
+                load_group(part, 0);
+#pragma unroll 1
+                for (int c = part; c < nchunks; c += n_own) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = 0.0f;
+#pragma unroll 1
+                    for (int i0 = 0; i0 < nparts - 1; i0 += DP) {
+                        if (i0 > 0) load_group(c, i0);
 #pragma unroll
                         for (int g = 0; g < DP; ++g) {
-                            const float4* src = reinterpret_cast<const float4*>(
-                                P.partials + static_cast<size_t>(min(c_first + q0 + g, c_last)) * slot_floats);
+                            if (i0 + g == part) {  // this CTA's own part comes before part `part` + 1
+                                float own[16];
+                                tmem_ld_32x16(t_acc + static_cast<uint32_t>(c * 32 + half * 16), own);
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) a[g][j] = __ldcg(src + static_cast<size_t>(half * 4 + j) * kBM + rt);
-                        }
-#pragma unroll
-                        for (int g = 0; g < DP; ++g)
-                            if (g < qn) {
+                                for (int j = 0; j < 16; ++j) v[j] += own[j];
+                            }
+                            if (i0 + g < nparts - 1) {
 #pragma unroll
                                 for (int j = 0; j < 4; ++j) {
                                     v[4 * j] += a[g][j].x;
@@ -867,96 +922,58 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
                                     v[4 * j + 3] += a[g][j].w;
                                 }
                             }
-                    }
-                    if (stop) break;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        v[4 * j] += al[j].x;
-                        v[4 * j + 1] += al[j].y;
-                        v[4 * j + 2] += al[j].z;
-                        v[4 * j + 3] += al[j].w;
-                    }
-                } else {
-                    tmem_ld_32x16(t_acc + static_cast<uint32_t>(c * 32 + half * 16), v);  // own (first) k-range
-                }
-                // a wide residual tile's old rows of this chunk, loaded while its parts arrive
-                float xw[kEpiGroup];
-                if constexpr (EPI == EPI_RESID && WIDE) {
-                    const int xrow = mt * kBM + rt;
-#pragma unroll
-                    for (int u = 0; u < kEpiGroup; ++u) {
-                        const int xcol = nt * p.ntile + c * 32 + half * kEpiGroup + u;
-                        xw[u] = (xrow < p.M && xcol < p.N) ? __ldcg(ep.out + static_cast<size_t>(xcol) * ep.ld_out + xrow)
-                                                           : 0.0f;
-                    }
-                }
-                for (int q = 1; !direct && q < nparts; ++q, ++si) {
-                    const int sl = si & (nsl - 1);
-                    mbar_wait(redbar + sl, (es.red_phase >> sl) & 1u, s_abort, status);
-                    es.red_phase ^= 1u << sl;
-                    if (threadIdx.x == 64) inflight &= ~(1u << sl);
-                    const float4* src = reinterpret_cast<const float4*>(red_stage + static_cast<size_t>(sl) * slice_bytes);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float4 a = src[(half * 4 + j) * kBM + rt];
-                        v[4 * j] += a.x;
-                        v[4 * j + 1] += a.y;
-                        v[4 * j + 2] += a.z;
-                        v[4 * j + 3] += a.w;
-                    }
-                    if (named_bar_any(1, kEpiThreads, *s_abort != 0)) {  // the slot is free again (or the launch failed)
-                        stop = true;
-                        break;
-                    }
-                    if (ew == 0 && si + nsl < nslices) issue(si + nsl);
-                }
-                if (stop) break;
-                if (tr && threadIdx.x == 64 && c == 0) {
-                    tr[kTrTicket] = global_ns();
-                    tr[kTrReduced] = global_ns();
-                    tr[kTrIsLast] = 1;
-                }
-                // the compact epilogue on the sum in registers (the residual's first pass leaves the
-                // new residual in the still owned accumulator, for the second)
-                epilogue_c32<EPI, kPass1>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
-                                          t_acc + static_cast<uint32_t>(c * 32),
-                                          t_x ? t_x + static_cast<uint32_t>(c * 32) : 0u, esm, e, half, quarter, lane,
-                                          status, v, (EPI == EPI_QKV && direct) ? &qpre : nullptr,
-                                          EPI == EPI_RESID && WIDE ? xw : nullptr);
-            }
-            if (threadIdx.x == 64) {
-                if (stop) {  // let copies in flight land before the shared memory is released
-                    const long long t0 = spin_clock();
-                    for (int sl = 0; sl < nsl; ++sl)
-                        while ((inflight >> sl & 1u) && !mbar_try_wait(redbar + sl, (es.red_phase >> sl) & 1u) &&
-                               spin_clock() - t0 < kWaitLimitCycles) {
                         }
-                } else {
-                    for (int q = 1; q < nparts; ++q) flags[q] = 0;  // ready for the next launch
+                    }
+                    if (tr && threadIdx.x == 64 && c + n_own >= nchunks) {
+                        tr[kTrReduced] = global_ns();
+                        tr[kTrIsLast] = 1;
+                    }
+                    if (c + n_own < nchunks) load_group(c + n_own, 0);
+                    if constexpr (EPI == EPI_RESID) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) v[j] += xw[j];
+                        if (c + n_own < nchunks) load_x(mt, nt, c + n_own);
+                    }
+                    epilogue_c32<EPI, kPass1, true>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
+                                              t_acc + static_cast<uint32_t>(c * 32), 0u, esm, e, half, quarter, lane,
+                                              status, v, nullptr, EPI == EPI_RESID, es.buf);
+                    es.buf ^= 1;
                 }
-            }
-            if (stop) {
-                cp_async_wait<0>();
-                return;
             }
         }
         if (tr && threadIdx.x == 64) tr[kTrEpiPass1] = global_ns();
-        if (finisher && P.done) {  // publish the finished tile to the next phase's operand producer
+        // A wide split tile's owners count themselves in on its word 31 (low byte: first passes,
+        // above it: second passes); the one whose count completes a pass publishes the tile
+        // (its acquire of the others' counts, then its release, order their stores too), and
+        // after the last pass leaves the words ready for the next launch.
+        constexpr bool two_pass = EPI == EPI_RESID;
+        auto publish = [&](int* done, int shift, bool last_pass) {  // thread 64, after the owner's barrier
+            if (WIDE && reducer && n_own > 1 &&
+                (atom_acq_rel_add(flags + kOwnerCount, 1 << shift) >> shift & 0xff) != n_own - 1)
+                return;
+            if (done) st_release(&done[mt * p.n_tiles + nt], tag);
+            if (WIDE && reducer && last_pass) {
+                for (int q = 0; q <= c_last - c_first; ++q) flags[q] = 0;
+                flags[kOwnerCount] = 0;
+            }
+        };
+        if (finisher && (P.done || (WIDE && reducer))) {  // publish the finished tile to the next phase's operand producer
             named_bar(1, kEpiThreads);
             if (threadIdx.x == 64) {
-                st_release(&P.done[mt * p.n_tiles + nt], tag);
+                publish(P.done, 0, !two_pass);
                 if (tr) tr[kTrPublished] = global_ns();
             }
         }
-        if constexpr (EPI == EPI_RESID) {
+        if constexpr (two_pass) {
             if (finisher) {  // then the fp32 residual and the RMSNorm sums, for the later phases' epilogues
-                for (int c = 0; c < nchunks; ++c)
+#pragma unroll 1
+                for (int c = WIDE && reducer ? part : 0; c < nchunks; c += WIDE && reducer ? n_own : 1)
                     epilogue_c32<EPI, 2>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
                                          t_acc + static_cast<uint32_t>(c * 32), 0u, esm, e, half, quarter,
                                          lane, status);
-                if (P.done2) {
+                if (P.done2 || (WIDE && reducer)) {
                     named_bar(1, kEpiThreads);
-                    if (threadIdx.x == 64) st_release(&P.done2[mt * p.n_tiles + nt], tag);
+                    if (threadIdx.x == 64) publish(P.done2, 8, true);
                 }
             }
         }
@@ -970,30 +987,28 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
         }
         it = tile * p.kb + k_hi;
     }
-    cp_async_wait<0>();
     if (tr && threadIdx.x == 64) tr[kTrEpiDone] = global_ns();
 }
 
 template <int DP, bool WIDE>
-__device__ __forceinline__ void chain_epilogue_dispatch(const ChainArgs& ca, int ph, int tag, uint8_t* red_stage,
-                                                        uint64_t* tfull, uint64_t* tempty, uint64_t* redbar,
+__device__ __forceinline__ void chain_epilogue_dispatch(const ChainArgs& ca, int ph, int tag, uint64_t* tfull, uint64_t* tempty,
                                                         volatile int* s_abort, uint32_t tmem_base, const EpiSmem& esm,
                                                         ChainEpiState& es) {
     switch (ca.ph[ph].epi) {
         case EPI_F32:
-            chain_phase_epilogue<EPI_F32, DP, WIDE>(ca, ph, tag, red_stage, tfull, tempty, redbar, s_abort, tmem_base, esm, es);
+            chain_phase_epilogue<EPI_F32, DP, WIDE>(ca, ph, tag, tfull, tempty, s_abort, tmem_base, esm, es);
             break;
         case EPI_RESID:
-            chain_phase_epilogue<EPI_RESID, DP, WIDE>(ca, ph, tag, red_stage, tfull, tempty, redbar, s_abort, tmem_base, esm, es);
+            chain_phase_epilogue<EPI_RESID, DP, WIDE>(ca, ph, tag, tfull, tempty, s_abort, tmem_base, esm, es);
             break;
         case EPI_QKV:
-            chain_phase_epilogue<EPI_QKV, DP, WIDE>(ca, ph, tag, red_stage, tfull, tempty, redbar, s_abort, tmem_base, esm, es);
+            chain_phase_epilogue<EPI_QKV, DP, WIDE>(ca, ph, tag, tfull, tempty, s_abort, tmem_base, esm, es);
             break;
         case EPI_SWIGLU:
-            chain_phase_epilogue<EPI_SWIGLU, DP, WIDE>(ca, ph, tag, red_stage, tfull, tempty, redbar, s_abort, tmem_base, esm, es);
+            chain_phase_epilogue<EPI_SWIGLU, DP, WIDE>(ca, ph, tag, tfull, tempty, s_abort, tmem_base, esm, es);
             break;
         default:
-            chain_phase_epilogue<EPI_LMHEAD, DP, WIDE>(ca, ph, tag, red_stage, tfull, tempty, redbar, s_abort, tmem_base, esm, es);
+            chain_phase_epilogue<EPI_LMHEAD, DP, WIDE>(ca, ph, tag, tfull, tempty, s_abort, tmem_base, esm, es);
             break;
     }
 }
@@ -1063,7 +1078,7 @@ __device__ __forceinline__ void q4_expand_tmem(const uint8_t* __restrict__ raw, 
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-template <bool Q4>
+template <bool Q4, bool WIDE>
 __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
     k_chain(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainArgs ca) {
     extern __shared__ uint8_t smem_raw[];
@@ -1084,22 +1099,22 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
     uint8_t* sA = smem;
     uint8_t* sB = sA + (a_tm ? 0 : static_cast<size_t>(S) * kABytes);
     uint8_t* sRaw = sB + static_cast<size_t>(SB) * b_slot;  // 4-bit weight tiles (Q4)
-    uint8_t* red_stage = sRaw + static_cast<size_t>(R) * raw_slot;
-    float* tail = reinterpret_cast<float*>(red_stage + ca.red_bytes + ca.stg_bytes);
+    uint8_t* stg = sRaw + static_cast<size_t>(R) * raw_slot;  // the epilogue's output staging
+    float* tail = reinterpret_cast<float*>(stg + (WIDE ? 2 : 1) * kStgBytes);
     EpiSmem esm;
     esm.rs = tail;
     esm.red = tail + 256;
     esm.kvs = reinterpret_cast<int*>(tail + 256 + 1024);
     esm.theta = tail + 256 + 1024 + 256;
-    esm.stg = ca.stg_bytes ? red_stage + ca.red_bytes : red_stage;
-    float* after = tail + 256 + 1024 + 256 + 128;
+    esm.stg = stg;
+    esm.step = tail + 256 + 1024 + 256 + 128;
+    float* after = tail + kTailFloats;
     uint64_t* full = reinterpret_cast<uint64_t*>(after);
     uint64_t* empty = full + S;
     uint64_t* tfull = empty + S;
     uint64_t* tempty = tfull + 2;
     uint64_t* drain = tempty + 2;
-    uint64_t* redbar = drain + 1;  // the partial staging slots (one or two)
-    uint64_t* rfull = redbar + 2;  // raw 4-bit tiles (Q4): arrived / read
+    uint64_t* rfull = drain + 1;  // raw 4-bit tiles (Q4): arrived / read
     uint64_t* rempty = rfull + R;
     uint64_t* bfull = rempty + R;  // operand tiles of the 4-bit kernel: arrived / consumed
     uint64_t* bempty = bfull + (Q4 ? SB : 0);
@@ -1132,8 +1147,6 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
             mbar_init(&tempty[a], kEpiThreads);
         }
         mbar_init(drain, 1);
-        mbar_init(&redbar[0], 1);
-        mbar_init(&redbar[1], 1);
         *s_abort = 0;
         int rows = -1;
         if (ca.dyn_rows) {
@@ -1431,16 +1444,15 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
         for (int ph = 0; ph < ca.n_phases && !stop; ++ph) {
             const GemmPlan p = phase_plan(ca.ph[ph], urows);
             if (static_cast<int>(blockIdx.x) >= p.grid) continue;
-            const long long it0 = range_begin(blockIdx.x, p.total, p.grid);
-            const long long it1 = range_begin(blockIdx.x + 1, p.total, p.grid);
+            const int it0 = static_cast<int>(range_begin(blockIdx.x, p.total, p.grid));
+            const int it1 = static_cast<int>(range_begin(blockIdx.x + 1, p.total, p.grid));
             unsigned long long* tr =
                 (leader && ca.ph[ph].ep.trace) ? ca.ph[ph].ep.trace + static_cast<size_t>(blockIdx.x) * kTrSlots : nullptr;
             bool first = true;
-            for (long long it = it0; it < it1;) {
-                const long long tile = it / p.kb;
-                const int k_lo = static_cast<int>(it - tile * p.kb);
-                const long long tend = (tile + 1) * p.kb;
-                const int k_hi = static_cast<int>((it1 < tend ? it1 : tend) - tile * p.kb);
+            for (int it = it0; it < it1;) {
+                const int tile = it / p.kb;
+                const int k_lo = it - tile * p.kb;
+                const int k_hi = min(it1 - tile * p.kb, p.kb);
                 if (__any_sync(0xffffffffu, *s_abort != 0) ||
                     !__all_sync(0xffffffffu, mbar_wait(&tempty[acc], acc_phase ^ 1u, s_abort, status))) {
                     stop = true;
@@ -1523,18 +1535,12 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
         // ---------------------------------------------------------- epilogue
         pdl_wait();
         const int tag = chain_tag(ca);
-        ChainEpiState es{0, 0u, 0u};
+        ChainEpiState es{0, 0u, 0};
         // split 32-token tiles: parts whose rows are loaded into registers at once (the 4-bit
         // kernel's smaller register budget takes two)
-        constexpr int kDP = Q4 ? 2 : 4;
-        for (int ph = 0; ph < ca.n_phases; ++ph) {  // on abort every phase returns at its first barrier
-            if (ca.ntile == 32)
-                chain_epilogue_dispatch<kDP, false>(ca, ph, tag, red_stage, tfull, tempty, redbar, s_abort, tmem_base,
-                                                    esm, es);
-            else
-                chain_epilogue_dispatch<kDP, true>(ca, ph, tag, red_stage, tfull, tempty, redbar, s_abort, tmem_base,
-                                                   esm, es);
-        }
+        constexpr int kDP = WIDE ? (Q4 ? 1 : 2) : (Q4 ? 2 : 4);
+        for (int ph = 0; ph < ca.n_phases; ++ph)  // on abort every phase returns at its first barrier
+            chain_epilogue_dispatch<kDP, WIDE>(ca, ph, tag, tfull, tempty, s_abort, tmem_base, esm, es);
     }
 
     tc_fence_before();
@@ -1570,6 +1576,7 @@ GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi) {
     const long long min_iters = (p.kb + 29) / 30;
     if (p.grid > p.total / min_iters) p.grid = static_cast<int>(p.total / min_iters);
     if (p.grid < 1) p.grid = 1;
+    p.slots = p.ntile > 32 ? 2 : 1;
     p.pdl = true;
     return p;
 }
@@ -1656,17 +1663,10 @@ bool chain_plan(ChainArgs& ca, int smem_budget) {
     ca.grid = grid;
     ca.ntile = ntile;
     ca.acc_cols = c32 ? 32 : pow2ceil(ntile);
-    ca.x_cols = ntile <= 128 ? ntile : 0;  // staged residual (none for 256-token tiles: TMEM is full)
+    ca.x_cols = c32 ? ntile : 0;  // staged old residual (wider tiles read it with the parts)
     ca.tmem_cols = pow2ceil(2 * ca.acc_cols + ca.x_cols);
-    // Partial slices staged for the finisher of a split tile of several 32-token chunks: two in
-    // flight, one for 256-token tiles (their ring needs the room: the tensor cores keep busy
-    // with 4 stages of 256 tokens, not with 3); for 32-token chains, whose finishers load the
-    // parts straight into registers, one slot that is the output staging.
-    ca.red_bytes = (c32 || ntile > 128 ? 1 : 2) * 32 * kBM * 4;
     const int stage_bytes = static_cast<int>(kABytes) + ntile * kBK * 2;
-    // tiles of more than one 32-token chunk: their own 8 KB for the bf16 output staging
-    ca.stg_bytes = c32 ? 0 : 32 * kBM * 2;
-    const int fixed0 = 1024 + (256 + 1024 + 256 + 128) * 4 + ca.red_bytes + ca.stg_bytes + 7 * 8 + 16;
+    const int fixed0 = 1024 + kTailFloats * 4 + (c32 ? 1 : 2) * kStgBytes + 5 * 8 + 16;
     if (ca.q4) {
         // 4-bit weights (480 threads: no room beside the CTA for another one, so all of shared
         // memory): raw 4.5 KB tiles, a few bf16 A stages the dequantizers fill (in tensor memory
@@ -1710,24 +1710,22 @@ bool chain_plan(ChainArgs& ca, int smem_budget) {
     ca.b_stages = 0;
     ca.a_tmem = 0;
     ca.a_col0 = 0;
-    // wide residual tiles read the old residual from global memory (a warp's 32 rows of a token
-    // are one 128-byte line), not from a staged copy: the ring keeps the room
-    const int fixed = fixed0;
-    int st = (smem_budget - fixed) / (stage_bytes + 16);
+    int st = (smem_budget - fixed0) / (stage_bytes + 16);
     if (st > 32) st = 32;
     if (st < 2) return false;
     ca.stages = st;
-    ca.smem = static_cast<size_t>(fixed) + static_cast<size_t>(st) * (stage_bytes + 16);
+    ca.smem = static_cast<size_t>(fixed0) + static_cast<size_t>(st) * (stage_bytes + 16);
     return ca.smem <= static_cast<size_t>(kFullSmem);
 }
 
 cudaError_t chain_init_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_chain<false>),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kFullSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_chain<true>),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kFullSmem);
-    return e;
+    const void* ks[4] = {reinterpret_cast<const void*>(k_chain<false, false>),
+                         reinterpret_cast<const void*>(k_chain<false, true>),
+                         reinterpret_cast<const void*>(k_chain<true, false>),
+                         reinterpret_cast<const void*>(k_chain<true, true>)};
+    for (const void* k : ks)
+        if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFullSmem)) return e;
+    return cudaSuccess;
 }
 
 cudaError_t chain_launch(const ChainMaps& maps, const ChainArgs& ca, cudaStream_t st, bool pdl) {
@@ -1743,9 +1741,9 @@ cudaError_t chain_launch(const ChainMaps& maps, const ChainArgs& ca, cudaStream_
         for (int i = 0; i < ca.n_phases; ++i)
             if (!ca.ph[i].w_tiles) return cudaErrorInvalidValue;
         if (ca.raw_stages < 2 || ca.raw_stages > 32 || ca.b_stages < 2 || ca.b_stages > 32) return cudaErrorInvalidValue;
-        return launch_k(k_chain<true>, dim3(ca.grid), dim3(kChainThreadsQ4), ca.smem, st, pdl, maps, ca);
+        return launch_k(ca.ntile == 32 ? k_chain<true, false> : k_chain<true, true>, dim3(ca.grid), dim3(kChainThreadsQ4), ca.smem, st, pdl, maps, ca);
     }
-    return launch_k(k_chain<false>, dim3(ca.grid), dim3(kChainThreads), ca.smem, st, pdl, maps, ca);
+    return launch_k(ca.ntile == 32 ? k_chain<false, false> : k_chain<false, true>, dim3(ca.grid), dim3(kChainThreads), ca.smem, st, pdl, maps, ca);
 }
 
 }  // namespace dllm

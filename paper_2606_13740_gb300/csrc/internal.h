@@ -94,11 +94,12 @@ struct GemmPlan {
     int m_tiles, n_tiles, kb;
     long long total;     // m_tiles * n_tiles * kb iterations of 64-wide K blocks
     int grid;            // CTAs (stream-K partition of the iterations)
+    int slots;           // split partials a CTA may store: two let a wide tile's parts share its epilogue
     bool pdl;            // launch with programmatic dependent launch (the step's chain)
 };
 
 struct Scratch {
-    float* partials;     // [grid][ntile*128]: one split partial per CTA (gemm_partial_floats)
+    float* partials;     // [grid][slots][ntile*128]: split partials (gemm_partial_floats)
     int* counters;       // tile tickets, one per 128-byte line ([m_tiles*n_tiles][32]), zero between launches
     size_t partial_floats;
     int counter_len;
@@ -120,7 +121,7 @@ struct ChainPhase {
     // residual phases: done = the bf16 operand is written, done2 = also the fp32 residual and
     // the RMSNorm sums (what the later phases' epilogues read); null: done covers both
     int* done2;
-    float* partials;     // [grid][ntile*128] split partials (a CTA contributes to at most one tile per phase)
+    float* partials;     // [grid][p.slots][ntile*128] split partials
     int* tickets;        // [m_tiles*n_tiles][32], zero between launches
     // non-null: the weights are stored tile-major (tiled_index) and each 16 KB tile arrives with
     // one contiguous bulk copy; null: row-major [M][K] through the chain's tensor map.  In a
@@ -131,9 +132,7 @@ struct ChainPhase {
 struct ChainArgs {
     int n_phases;
     int grid, stages, ntile, acc_cols, tmem_cols;
-    int red_bytes;       // shared staging for split partials
     int x_cols;          // TMEM columns for the staged old residual (0: none)
-    int stg_bytes;       // the epilogue's own output staging (0: it shares the partial staging)
     size_t smem;
     const int* epoch;    // device step counter; tag = *epoch * tag_mul + tag_add (null: tag = tag_add)
     int tag_mul, tag_add;
@@ -162,8 +161,7 @@ struct ChainMaps {
     CUtensorMap w[kMaxPhases];
     CUtensorMap x[kMaxPhases];
 };
-// Fills grid, stages, ntile, acc_cols, x_cols, stg_bytes, tmem_cols, red_bytes and
-// smem from the phases' plans for a shared-memory budget (bytes, <= 227 KB).  False if the
+// Fills grid, stages, ntile, acc_cols, x_cols, tmem_cols and smem from the phases' plans for a shared-memory budget (bytes, <= 227 KB).  False if the
 // phases do not share one token tiling.
 bool chain_plan(ChainArgs& ca, int smem_budget);
 constexpr int kChainSmemFull = 227 * 1024;    // one CTA per SM, deepest ring
@@ -174,10 +172,10 @@ cudaError_t chain_init_attrs();
 // Tiling of one projection: token tiles of at most 256 (multiples of 32), 128 weight rows
 // per tile, 64-wide k-blocks, grid = min(iterations, grid_max).
 GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi);
-// Split-partial floats a single-projection launch of plan p needs (a CTA contributes to at most
-// one split tile, so one ntile x 128 slot per CTA); gemm_launch rejects a smaller Scratch.
+// Split-partial floats a single-projection launch of plan p needs (ntile x 128 per slot);
+// gemm_launch rejects a smaller Scratch.
 inline size_t gemm_partial_floats(const GemmPlan& p) {
-    return static_cast<size_t>(p.grid) * static_cast<size_t>(p.ntile) * 128;
+    return static_cast<size_t>(p.grid) * static_cast<size_t>(p.slots) * static_cast<size_t>(p.ntile) * 128;
 }
 bool make_tmap_bf16(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows);
 cudaError_t gemm_launch(int epi, const GemmPlan& p, const CUtensorMap& tmW, const CUtensorMap& tmX,

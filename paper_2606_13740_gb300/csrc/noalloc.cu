@@ -67,6 +67,7 @@ extern "C" int dllm_op_gemm_noalloc(const void* W, const void* X, float* D, int 
         return noalloc_fail(DLLM_ECUDA, "device query failed");
     GemmPlan p = gemm_plan(M, N, K, (grid > 0 && grid < sms) ? grid : sms, EPI_F32);
     p.pdl = false;
+    p.slots = 1;  // one partial a CTA: twice the CTAs fit the array
     // the split partials sit behind the tickets; gemm_partial_floats is the bound gemm_launch
     // checks, so the grid that fits is the one whose partials fit the rest of the array
     GemmPlan one = p;
@@ -79,6 +80,7 @@ extern "C" int dllm_op_gemm_noalloc(const void* W, const void* X, float* D, int 
         if (grid > 0) return noalloc_fail(DLLM_ECAPACITY, "grid too large for the static scratch");
         p = gemm_plan(M, N, K, static_cast<int>(cap_ctas), EPI_F32);  // auto grid: shrink to fit
         p.pdl = false;
+        p.slots = 1;
     }
     if (gemm_init_attrs() != cudaSuccess) return noalloc_fail(DLLM_ECUDA, "attribute setup failed");
     CUtensorMap tw, tx;

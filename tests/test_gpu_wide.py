@@ -1,0 +1,57 @@
+"""Split tiles of wide token tiles at the sizes where their bookkeeping can go wrong, against the same
+sums in 64 bits."""
+import numpy as np
+import pytest
+
+import oracle as O
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2606_13740_gb300 as p
+    p.lib()
+    return p
+
+
+def _bf16(g, *shape, sigma=1.0):
+    return (torch.randn(*shape, generator=g, dtype=torch.float32) * sigma).to(torch.bfloat16).cuda()
+
+
+# (M, N, K, grid): one tile of 31 parts; more parts than chunks; two parts (one finisher); three (two
+# finishers, uneven chunks); two chunks; several token tiles; whole tiles beside split ones; a grid
+# that cuts no tile; one part per k-block
+@pytest.mark.parametrize("M,N,K,grid", [
+    (128, 250, 18944, 0), (128, 64, 18944, 0), (1024, 251, 4096, 0), (12288, 256, 1024, 0), (256, 96, 640, 5),
+    (384, 33, 1088, 0), (4096, 96, 4096, 0), (640, 515, 2048, 0), (24576, 65, 512, 0), (512, 200, 640, 4),
+    (200, 129, 64, 0), (130, 40, 192, 0),
+])
+def test_wide_split_tiles(pkg, M, N, K, grid):
+    g = torch.Generator().manual_seed(M + N + K)
+    W, X = _bf16(g, M, K, sigma=0.05), _bf16(g, N, K)
+    D = pkg.dllm_op_gemm(W, X, M, N, K, grid=grid)
+    w, x = W.double(), X.double()
+    # fp32 sums of exact products: rounding errors of random sign, a few 2^-24 sqrt(K) of the terms'
+    # size, i.e. of the norms' product over sqrt(K) (1e-5 of that product is 160 x 2^-24)
+    tol = 1e-5 * x.norm(dim=1)[:, None] * w.norm(dim=1)[None, :]
+    assert bool(((D.double() - x @ w.T).abs() <= tol).all())
+    assert torch.equal(D, pkg.dllm_op_gemm(W, X, M, N, K, grid=grid))
+
+
+@pytest.mark.parametrize("V,N,d", [(1024, 251, 4096), (512, 96, 2048), (4096, 64, 512)])
+def test_wide_head_split_tiles(pkg, V, N, d):
+    g = torch.Generator().manual_seed(V + N)
+    W, X = _bf16(g, V, d, sigma=0.02), _bf16(g, N, d)
+    cur = torch.randint(0, V - 1, (N,), generator=g, dtype=torch.int32).cuda()
+    x0, conf, tc, lg = pkg.dllm_op_lmhead(W, X, cur, V, N, d, V - 1, want_logits=True)
+    ref = (X.double() @ W.double().T).cpu().numpy()
+    assert np.abs(lg.cpu().numpy() - ref).max() <= 1e-4 * np.abs(ref).max()
+    x0, conf, tc, cur = (t.cpu().numpy() for t in (x0, conf, tc, cur))
+    for n in range(N):
+        rx0, rconf, rtc, margin = O.decide(ref[n].astype(np.float32), V - 1, cur[n])
+        assert margin <= 1e-3 or x0[n] == rx0
+        assert abs(conf[n] - rconf) <= 1e-3 * rconf and abs(tc[n] - rtc) <= 1e-3 * rtc + 1e-12
