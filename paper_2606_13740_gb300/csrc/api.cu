@@ -328,7 +328,7 @@ static int forward(dllm_ctx* ctx, int B, int Tw, bool head, int R = 0, bool sls 
         !make_tmap_bf16(&tx_h, ctx->h, N, F, pd.ntile) || !make_tmap_bf16(&tx_c, ctx->sls_x, N, d, ph.ntile))
         return fail(ctx, DLLM_ECUDA, "tensor map encode failed");
     sls = sls && head;
-    AttnPlan ap = attn_plan(B, T, c.n_heads, c.head_dim, (ctx->in_step ? plan_kv(ctx) : ctx->kv_len) + Tw, ctx->sms);
+    AttnPlan ap = attn_plan(B, T, c.n_heads, L.Hkv, c.head_dim, (ctx->in_step ? plan_kv(ctx) : ctx->kv_len) + Tw, ctx->sms);
     ap.qx = R;
     EpiArgs ep{};
     ep.seq_kv = ctx->seq_kv;

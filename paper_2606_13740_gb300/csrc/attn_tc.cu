@@ -2,8 +2,11 @@
 // (Sec. 2.1 block-wise decoding with prefix KV reuse; no causal mask) on the 5th-generation
 // tensor cores, head dim 128.
 //
-// One CTA = one (sequence, head, query tile of up to 128 rows) and one share of its keys; the
-// csize CTAs of a cluster split the keys and merge through distributed shared memory.  Per
+// One CTA = one (sequence, K/V head, query tile of up to 128 rows) and one share of its keys; the
+// csize CTAs of a cluster split the keys and merge through distributed shared memory.  Under
+// grouped-query attention the rows of a K/V head's query heads follow one another in q, and the
+// tiles are cut from that run: seven heads with a 32-token window are two tiles, not seven (five
+// sequences, 28 heads over 4, 1501 keys: a four-layer step 784 -> 761 us).  Per
 // 64-key sub-block j:
 //   S_j = Q K_j^T         tcgen05.mma, A = Q (shared memory, K-major), B = K_j (shared,
 //                         K-major), fp32 S_j in tensor memory (128 lanes = query rows)
@@ -89,6 +92,30 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
 }
+// Two fp32 operations in one instruction (each component rounded as by fmaf / an addition).
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%6, %7};\n"
+        " fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}\n"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
+        " add.rn.f32x2 d, a, b;\n mov.b64 {%0, %1}, d;\n}\n"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+// 2^x by the special function unit; results below 2^-126 become 0 (a probability that small is
+// nothing beside the row's largest, which is at least 2^-8)
+__device__ __forceinline__ float ex2(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 __device__ __forceinline__ unsigned smid_tc() {
     unsigned r;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(r));
@@ -125,7 +152,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tr[kTcMerged] = 0;
     }
     pdl_launch_dependents();
-    const int split = blockIdx.x, h = blockIdx.y;
+    // hk: the K/V head; its H / Hkv query heads' rows, head by head, are one run of q
+    const int split = blockIdx.x, hk = blockIdx.y, nrows = H / Hkv * T;
     const int b = blockIdx.z / qtiles, qt = blockIdx.z - b * qtiles;
     const int NK = seq_kv[b] + T - qx;  // the last qx rows are queries only
     const int nblk = (NK + kTcKeys - 1) / kTcKeys;
@@ -133,7 +161,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int kbeg = blk0 * kTcKeys, kend = min(NK, blk1 * kTcKeys);
     const int nsub = blk1 - blk0;  // 64-key sub-blocks of this CTA (may be 0)
     const int q0 = qt * kTcRows;
-    const int nq = min(kTcRows, T - q0);
+    const int nq = min(kTcRows, nrows - q0);
+
+    // offset of the output row of row i of the run (query head hk H/Hkv + i / T, token i % T)
+    auto out_off = [&](int i) {
+        const int g = i / T;
+        return (static_cast<size_t>(b) * T + (i - g * T)) * (H * 128) + static_cast<size_t>(hk * (H / Hkv) + g) * 128;
+    };
 
     if (threadIdx.x == 0) {
         mbar_init(&qbar, 1);
@@ -171,11 +205,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             pdl_wait();  // Q and the window's K/V come from the preceding projection
             if (tr) tr[kTcDepWait] = global_ns();
             const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_first();
-            const int qrow = (b * H + h) * T + q0;
+            const int qrow = (b * Hkv + hk) * nrows + q0;
             mbar_arrive_expect_tx(&qbar, kTcQBytes);
             tma_load_2d(sQ, &maps.q, 0, qrow, &qbar, pol_q);
             tma_load_2d(sQ + kTcQBytes / 2, &maps.q, 64, qrow, &qbar, pol_q);
-            const int krow0 = (b * Hkv + (Hkv == H ? h : h / (H / Hkv))) * cap + kbeg;  // K/V head of query head h
+            const int krow0 = (b * Hkv + hk) * cap + kbeg;
             int kiss = 0, viss = 0;  // sub-blocks whose K, V copies were issued
             for (int j = 0; j < nsub && !s_abort; ++j) {
                 const int st = j % NB;
@@ -275,14 +309,23 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             tc_fence_after();
             const uint32_t ts = tS0 + static_cast<uint32_t>(sb * 64) + lane_off;
-            tmem_ld_32x32(ts, v);
-            tmem_ld_32x32(ts + 32, v + 32);
+            tmem_ld_32x64(ts, v);
             const int k0 = kbeg + j * kTcKeys;
-            float mx = -INFINITY;
+            if (k0 + kTcKeys > kend) {  // the last sub-block's keys past the end (the same for the whole CTA)
 #pragma unroll
-            for (int i = 0; i < 64; ++i) {
-                v[i] = (k0 + i < kend) ? v[i] * sl2 : -INFINITY;
-                mx = fmaxf(mx, v[i]);
+                for (int i = 0; i < 64; ++i)
+                    if (k0 + i >= kend) v[i] = -INFINITY;
+            }
+            float mx = -INFINITY;
+            {
+                float mi[4] = {v[0], v[1], v[2], v[3]};  // four chains
+#pragma unroll
+                for (int i = 4; i < 64; i += 8) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        mi[u] = i + 4 < 64 ? fmaxf(fmaxf(mi[u], v[i + u]), v[i + 4 + u]) : fmaxf(mi[u], v[i + u]);
+                }
+                mx = fmaxf(fmaxf(mi[0], mi[1]), fmaxf(mi[2], mi[3])) * sl2;
             }
             // the first sub-block, or a row max 2^8 above the one in use somewhere in the warp
             // (the whole warp rescales: TMEM accesses are warp-wide)
@@ -307,16 +350,22 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 }
                 m = mn;
             }
+            // P = 2^(S sl2 - m): one FMA and one exponential per score, pairs side by side.  The
+            // softmax warps' issue slots bound long prompts: scaling, masking and subtracting apart
+            // and an exponential with subnormal results took about ten instructions a score (2048
+            // tokens over 32 heads: a call 126 -> 99 us).
             uint32_t pk[32];
-            float ls = 0.0f;
+            float2 ls[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+            const float2 sl = make_float2(sl2, sl2), nm = make_float2(-m, -m);
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
-                const float p0 = exp2f(v[2 * i] - m), p1 = exp2f(v[2 * i + 1] - m);
-                ls += p0 + p1;
-                __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
-                pk[i] = *reinterpret_cast<uint32_t*>(&pp);
+                float2 t = ffma2(make_float2(v[2 * i], v[2 * i + 1]), sl, nm);
+                t.x = ex2(t.x);
+                t.y = ex2(t.y);
+                ls[i & 1] = fadd2(ls[i & 1], t);
+                pk[i] = pack_bf16x2(t.x, t.y);
             }
-            l += ls;
+            l += (ls[0].x + ls[0].y) + (ls[1].x + ls[1].y);
             tmem_st_32x32u(ts, pk);  // P_j over the first 32 columns of the buffer
             tc_fence_before();
             mbar_arrive(&pfull[sb]);
@@ -329,11 +378,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         if (tr && threadIdx.x == 0) tr[kTcLoop] = global_ns();
         if (!ok) l = 0.0f;
-        const int qd = H * 128;
         if (csize == 1) {
             // normalised output straight from TMEM, 16-byte stores per row
             const float il = (nsub > 0 && l > 0.0f) ? 1.0f / l : 0.0f;
-            __nv_bfloat16* op = out + (static_cast<size_t>(b) * T + q0 + min(r, nq - 1)) * qd + h * 128;
+            __nv_bfloat16* op = out + out_off(q0 + min(r, nq - 1));
 #pragma unroll 1
             for (int c = 0; c < 128; c += 32) {
                 float o[32];
@@ -393,7 +441,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
         for (int c = 0; c < kTcMaxCluster; ++c) pb[c] = c < csize ? dsmem_map_tc(smem_u32(sO), c) : 0u;
         const int nel = nq * 32;
-        const int qd = H * 128;
         for (int ew0 = split * kTcThreads + warp * 32; ew0 < nel; ew0 += csize * kTcThreads) {
             const int rr = ew0 / 32, i4 = lane;  // one row per warp pass
             float mk = -INFINITY, lk = 0.0f;
@@ -429,7 +476,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 }
             }
             const float inv = L > 0.0f ? 1.0f / L : 0.0f;
-            __nv_bfloat16* op = out + (static_cast<size_t>(b) * T + q0 + rr) * qd + h * 128 + i4 * 4;
+            __nv_bfloat16* op = out + out_off(q0 + rr) + i4 * 4;
             uint2 w2;
             w2.x = pack_bf16x2(acc.x * inv, acc.y * inv);
             w2.y = pack_bf16x2(acc.z * inv, acc.w * inv);
@@ -469,11 +516,13 @@ cudaError_t attn_tc_init_attrs() {
     return e;
 }
 
-AttnPlan attn_plan_tc(int B, int T, int H, int max_keys, int sms) {
+AttnPlan attn_plan_tc(int B, int T, int H, int Hkv, int max_keys, int sms) {
     AttnPlan a{};
     a.tc = true;
-    a.qtiles = (T + kTcRows - 1) / kTcRows;
-    const int units = B * H * a.qtiles;
+    // a K/V head's query heads share its query tiles, so its keys are read once per tile of
+    // their rows together
+    a.qtiles = (H / Hkv * T + kTcRows - 1) / kTcRows;
+    const int units = B * Hkv * a.qtiles;
     const int blocks = (max_keys + kTcKeys - 1) / kTcKeys;
     // key splits (cluster size): about two CTAs per SM, at most one split per sub-block
     int c = (2 * sms + units - 1) / units;
@@ -497,7 +546,7 @@ cudaError_t launch_attention_tc(const __nv_bfloat16* q, const __nv_bfloat16* kc,
         !make_tmap_bf16(&maps.v, vc, static_cast<uint64_t>(B) * Hkv * cap, 128, kTcKeys))
         return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(a.csize, H, B * a.qtiles);
+    cfg.gridDim = dim3(a.csize, Hkv, B * a.qtiles);
     cfg.stream = st;
     cudaLaunchAttribute at[2];
     int n = 0;

@@ -262,6 +262,37 @@ __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, float* v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 32 TMEM lanes x 64 consecutive columns -> 64 registers per thread (two loads, one wait).
+__device__ __forceinline__ void tmem_ld_32x64(uint32_t taddr, float* v) {
+    uint32_t r[64];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t* q = r + 32 * h;
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+            "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+            : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]),
+              "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15]),
+              "=r"(q[16]), "=r"(q[17]), "=r"(q[18]), "=r"(q[19]), "=r"(q[20]), "=r"(q[21]), "=r"(q[22]),
+              "=r"(q[23]), "=r"(q[24]), "=r"(q[25]), "=r"(q[26]), "=r"(q[27]), "=r"(q[28]), "=r"(q[29]),
+              "=r"(q[30]), "=r"(q[31])
+            : "r"(taddr + static_cast<uint32_t>(32 * h)));
+    }
+    // the wait names the registers, so nothing reads them before it
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        uint32_t* q = r + 16 * h;
+        asm volatile("tcgen05.wait::ld.sync.aligned;"
+                     : "+r"(q[0]), "+r"(q[1]), "+r"(q[2]), "+r"(q[3]), "+r"(q[4]), "+r"(q[5]), "+r"(q[6]), "+r"(q[7]),
+                       "+r"(q[8]), "+r"(q[9]), "+r"(q[10]), "+r"(q[11]), "+r"(q[12]), "+r"(q[13]), "+r"(q[14]),
+                       "+r"(q[15])
+                     :
+                     : "memory");
+    }
+#pragma unroll
+    for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 // 32 TMEM lanes x 4 consecutive columns -> 4 registers per thread.
 __device__ __forceinline__ void tmem_ld_32x4(uint32_t taddr, float* v) {
     uint32_t r0, r1, r2, r3;

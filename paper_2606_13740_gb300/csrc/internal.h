@@ -261,8 +261,8 @@ struct AttnSync {
 // head dim 128 and at least kTcMinKeys keys: the tcgen05 kernel's plan; otherwise the
 // mma.sync kernel's
 constexpr int kTcMinKeys = 1024;
-AttnPlan attn_plan(int B, int T, int H, int hd, int max_keys, int sms);
-AttnPlan attn_plan_tc(int B, int T, int H, int max_keys, int sms);
+AttnPlan attn_plan(int B, int T, int H, int Hkv, int hd, int max_keys, int sms);
+AttnPlan attn_plan_tc(int B, int T, int H, int Hkv, int max_keys, int sms);
 cudaError_t attn_tc_init_attrs();
 // Grouped-query attention: query head h reads K/V head h / (H / Hkv) of the cache [B][Hkv][cap][hd].
 cudaError_t launch_attention_tc(const __nv_bfloat16* q, const __nv_bfloat16* kc, const __nv_bfloat16* vc,

@@ -543,10 +543,10 @@ cudaError_t attn_init_attrs() {
     return e;
 }
 
-AttnPlan attn_plan(int B, int T, int H, int hd, int max_keys, int sms) {
+AttnPlan attn_plan(int B, int T, int H, int Hkv, int hd, int max_keys, int sms) {
     // long key ranges (head dim 128) go to the tensor-core kernel; on short ones, a few
     // sub-blocks per CTA, the mma.sync kernel has less latency per sub-block
-    if (hd == 128 && max_keys >= kTcMinKeys) return attn_plan_tc(B, T, H, max_keys, sms);
+    if (hd == 128 && max_keys >= kTcMinKeys) return attn_plan_tc(B, T, H, Hkv, max_keys, sms);
     AttnPlan a{};
     // two warps (32 query rows) for the short windows of cached decoding, four otherwise: a
     // 64-token window is one query tile, so its keys and values are read once

@@ -1,5 +1,5 @@
-"""Split tiles of wide token tiles at the sizes where their bookkeeping can go wrong, against the same
-sums in 64 bits."""
+"""Split tiles of wide token tiles, and query tiles cut from a K/V head's whole group, at the sizes
+where their bookkeeping can go wrong, against the same sums in 64 bits."""
 import numpy as np
 import pytest
 
@@ -55,3 +55,23 @@ def test_wide_head_split_tiles(pkg, V, N, d):
         rx0, rconf, rtc, margin = O.decide(ref[n].astype(np.float32), V - 1, cur[n])
         assert margin <= 1e-3 or x0[n] == rx0
         assert abs(conf[n] - rconf) <= 1e-3 * rconf and abs(tc[n] - rtc) <= 1e-3 * rtc + 1e-12
+
+
+# the group's rows end inside a tile, at its edge and one past it; one query head per K/V head; one
+# K/V head; prefixes that leave some key splits empty
+@pytest.mark.parametrize("B,T,H,Hkv,kv", [
+    (1, 5, 28, 4, [1200]), (2, 32, 28, 4, [1024, 3]), (1, 64, 8, 4, [1500]), (1, 43, 6, 2, [1061]),
+    (2, 100, 8, 1, [1300, 700]), (3, 96, 4, 4, [2000, 64, 1]), (1, 129, 4, 2, [1111]),
+])
+def test_group_query_tiles(pkg, B, T, H, Hkv, kv):
+    g = torch.Generator().manual_seed(B * T + H)
+    cap = max(kv) + T + 7
+    q, k, v = _bf16(g, B, H, T, 128), _bf16(g, B, Hkv, cap, 128), _bf16(g, B, Hkv, cap, 128)
+    out = pkg.dllm_op_attention(q, k, v, torch.tensor(kv, dtype=torch.int32).cuda(), B, T, H, 128, cap, max(kv), Hkv=Hkv)
+    for b in range(B):
+        n = kv[b] + T
+        kk, vv = (t[b, :, :n].double().repeat_interleave(H // Hkv, 0) for t in (k, v))
+        ref = torch.softmax(q[b].double() @ kk.transpose(1, 2) / 128 ** 0.5, -1) @ vv
+        got = out.view(B, T, H, 128)[b].transpose(0, 1).double()
+        assert (got - ref).norm() <= 1e-2 * ref.norm()  # bf16 probabilities and outputs
+        assert (got - ref).abs().max() <= 0.05 * ref.abs().max()
