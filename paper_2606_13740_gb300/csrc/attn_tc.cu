@@ -196,97 +196,123 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const uint32_t tmem = tslot;
     const uint32_t tO = tmem, tS0 = tmem + 128;
 
+    // The load and MMA warps run their loops whole, the outcomes of their waits voted, so that
+    // descriptors and addresses stay warp-uniform values, and one elected lane issues: a single
+    // lane running the loop alone took 50 to 80 cycles an instruction, which with 12 MMAs and four
+    // waits a sub-block bound the kernel (a prompt of 2048 tokens over 32 heads: 64 -> 54 us each in
+    // a batch of four; 16 x 64 rows over 4160 keys: a call 184 -> 174 us).
+    auto wait_all = [&](uint64_t* bar, uint32_t parity) {
+        return __all_sync(0xffffffffu, mbar_wait(bar, parity, &s_abort, status)) != 0;
+    };
     if (warp == 4) {
         // ------------------------------------------------ loads
-        if (lane == 0) {
+        const bool leader = elect_one();
+        if (leader) {
             tma_prefetch_desc(&maps.q);
             tma_prefetch_desc(&maps.k);
             tma_prefetch_desc(&maps.v);
-            pdl_wait();  // Q and the window's K/V come from the preceding projection
-            if (tr) tr[kTcDepWait] = global_ns();
-            const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_first();
+        }
+        pdl_wait();  // Q and the window's K/V come from the preceding projection
+        if (tr && lane == 0) tr[kTcDepWait] = global_ns();
+        const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_first();
+        if (leader && nsub > 0) {  // (a share without keys reads no Q and must not leave a copy in flight)
             const int qrow = (b * Hkv + hk) * nrows + q0;
             mbar_arrive_expect_tx(&qbar, kTcQBytes);
             tma_load_2d(sQ, &maps.q, 0, qrow, &qbar, pol_q);
             tma_load_2d(sQ + kTcQBytes / 2, &maps.q, 64, qrow, &qbar, pol_q);
-            const int krow0 = (b * Hkv + hk) * cap + kbeg;
-            int kiss = 0, viss = 0;  // sub-blocks whose K, V copies were issued
-            for (int j = 0; j < nsub && !s_abort; ++j) {
-                const int st = j % NB;
-                const uint32_t par = static_cast<uint32_t>((j / NB - 1) & 1);
-                if (j >= NB && !mbar_wait(&kempty[st], par, &s_abort, status)) break;
+        }
+        int krow = (b * Hkv + hk) * cap + kbeg;
+        int kiss = 0, viss = 0;  // sub-blocks whose K, V copies were issued
+        for (int j = 0; j < nsub; ++j, krow += kTcKeys) {
+            const int st = j % NB;
+            const uint32_t par = static_cast<uint32_t>((j / NB - 1) & 1);
+            uint8_t *dk = sK + st * kTcKVBytes, *dv = sV + st * kTcKVBytes;
+            if (j >= NB && !wait_all(&kempty[st], par)) break;
+            if (leader) {
                 mbar_arrive_expect_tx(&kfull[st], kTcKVBytes);
-                tma_load_2d(sK + st * kTcKVBytes, &maps.k, 0, krow0 + j * kTcKeys, &kfull[st], pol_kv);
-                tma_load_2d(sK + st * kTcKVBytes + kTcKVBytes / 2, &maps.k, 64, krow0 + j * kTcKeys, &kfull[st], pol_kv);
-                kiss = j + 1;
-                if (j >= NB && !mbar_wait(&vempty[st], par, &s_abort, status)) break;
+                tma_load_2d(dk, &maps.k, 0, krow, &kfull[st], pol_kv);
+                tma_load_2d(dk + kTcKVBytes / 2, &maps.k, 64, krow, &kfull[st], pol_kv);
+            }
+            kiss = j + 1;
+            if (j >= NB && !wait_all(&vempty[st], par)) break;
+            if (leader) {
                 mbar_arrive_expect_tx(&vfull[st], kTcKVBytes);
-                tma_load_2d(sV + st * kTcKVBytes, &maps.v, 0, krow0 + j * kTcKeys, &vfull[st], pol_kv);
-                tma_load_2d(sV + st * kTcKVBytes + kTcKVBytes / 2, &maps.v, 64, krow0 + j * kTcKeys, &vfull[st], pol_kv);
-                viss = j + 1;
+                tma_load_2d(dv, &maps.v, 0, krow, &vfull[st], pol_kv);
+                tma_load_2d(dv + kTcKVBytes / 2, &maps.v, 64, krow, &vfull[st], pol_kv);
             }
-            if (s_abort) {
-                // let the copies in flight land before the shared memory is released (one
-                // deadline for all)
-                const long long t0 = spin_clock();
-                while (!mbar_try_wait(&qbar, 0) && spin_clock() - t0 < kWaitLimitCycles) {
+            viss = j + 1;
+        }
+        if (leader && nsub > 0 && *const_cast<volatile int*>(&s_abort)) {
+            // let the copies in flight land before the shared memory is released (one
+            // deadline for all)
+            const long long t0 = spin_clock();
+            while (!mbar_try_wait(&qbar, 0) && spin_clock() - t0 < kWaitLimitCycles) {
+            }
+            for (int j = max(0, kiss - NB); j < kiss; ++j)
+                while (!mbar_try_wait(&kfull[j % NB], static_cast<uint32_t>((j / NB) & 1)) &&
+                       spin_clock() - t0 < kWaitLimitCycles) {
                 }
-                for (int j = max(0, kiss - NB); j < kiss; ++j)
-                    while (!mbar_try_wait(&kfull[j % NB], static_cast<uint32_t>((j / NB) & 1)) &&
-                           spin_clock() - t0 < kWaitLimitCycles) {
-                    }
-                for (int j = max(0, viss - NB); j < viss; ++j)
-                    while (!mbar_try_wait(&vfull[j % NB], static_cast<uint32_t>((j / NB) & 1)) &&
-                           spin_clock() - t0 < kWaitLimitCycles) {
-                    }
-            }
+            for (int j = max(0, viss - NB); j < viss; ++j)
+                while (!mbar_try_wait(&vfull[j % NB], static_cast<uint32_t>((j / NB) & 1)) &&
+                       spin_clock() - t0 < kWaitLimitCycles) {
+                }
         }
     } else if (warp == 5) {
         // ------------------------------------------------ MMA issue
-        if (lane == 0 && nsub > 0) {
+        if (nsub > 0) {
+            const bool leader = elect_one();
+            const uint32_t t_o = __shfl_sync(0xffffffffu, tmem, 0), t_s = t_o + 128;
             const uint32_t id_s = umma_idesc_bf16(kTcRows, kTcKeys);              // S = Q K^T
             const uint32_t id_o = umma_idesc_bf16(kTcRows, 128) | (1u << 16);    // O += P V, V MN-major
-            bool ok = mbar_wait(&qbar, 0, &s_abort, status);
+            const uint64_t qd = sw128_desc(smem_u32(sQ), 16, 1024), kd = sw128_desc(smem_u32(sK), 16, 1024);
+            const uint64_t vd = sw128_desc(smem_u32(sV), kTcKVBytes / 2, 1024);
             auto issue_s = [&](int j) {  // S_j into buffer j % 2
                 const int st = j % NB, sb = j % 2;
-                if (!mbar_wait(&kfull[st], static_cast<uint32_t>((j / NB) & 1), &s_abort, status)) return false;
+                if (!wait_all(&kfull[st], static_cast<uint32_t>((j / NB) & 1))) return false;
                 // buffer sb last held P_{j-2}: its P.V must be done
-                if (j >= 2 && !mbar_wait(&pvdone[sb], static_cast<uint32_t>(((j - 2) / 2) & 1), &s_abort, status))
-                    return false;
+                if (j >= 2 && !wait_all(&pvdone[sb], static_cast<uint32_t>(((j - 2) / 2) & 1))) return false;
                 tc_fence_after();
-                const uint32_t qa = smem_u32(sQ), ka = smem_u32(sK + st * kTcKVBytes);
+                if (leader) {
+                    const uint64_t kds = kd + static_cast<uint64_t>(st * (kTcKVBytes >> 4));
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {  // head dim 128 = 8 steps of 16
-                    const uint32_t off = static_cast<uint32_t>((kk >> 2) * (kTcQBytes / 2) + (kk & 3) * 32);
-                    const uint32_t offk = static_cast<uint32_t>((kk >> 2) * (kTcKVBytes / 2) + (kk & 3) * 32);
-                    umma_bf16(tS0 + static_cast<uint32_t>(sb * 64), sw128_desc(qa + off, 16, 1024),
-                              sw128_desc(ka + offk, 16, 1024), id_s, kk > 0 ? 1u : 0u);
+                    for (int kk = 0; kk < 8; ++kk)  // head dim 128 = 8 steps of 16
+                        umma_bf16(t_s + static_cast<uint32_t>(sb * 64),
+                                  qd + static_cast<uint64_t>(((kk >> 2) * (kTcQBytes / 2) + (kk & 3) * 32) >> 4),
+                                  kds + static_cast<uint64_t>(((kk >> 2) * (kTcKVBytes / 2) + (kk & 3) * 32) >> 4), id_s,
+                                  kk > 0 ? 1u : 0u);
+                    umma_commit(&sfull[sb]);
+                    umma_commit(&kempty[st]);
                 }
-                umma_commit(&sfull[sb]);
-                umma_commit(&kempty[st]);
+                __syncwarp();
                 return true;
             };
+            bool ok = wait_all(&qbar, 0);
             if (ok) ok = issue_s(0);
             for (int j = 0; j < nsub && ok; ++j) {
                 if (j + 1 < nsub && !issue_s(j + 1)) break;
                 const int st = j % NB, sb = j % 2;
-                if (!mbar_wait(&vfull[st], static_cast<uint32_t>((j / NB) & 1), &s_abort, status)) break;
-                if (!mbar_wait(&pfull[sb], static_cast<uint32_t>((j / 2) & 1), &s_abort, status)) break;
+                if (!wait_all(&vfull[st], static_cast<uint32_t>((j / NB) & 1))) break;
+                if (!wait_all(&pfull[sb], static_cast<uint32_t>((j / 2) & 1))) break;
                 tc_fence_after();
-                const uint32_t va = smem_u32(sV + st * kTcKVBytes);
+                if (leader) {
+                    const uint64_t vds = vd + static_cast<uint64_t>(st * (kTcKVBytes >> 4));
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)  // 64 keys = 4 steps of 16: P columns kk*8, V key groups 2kk
-                    umma_tmem_a(tO, tS0 + static_cast<uint32_t>(sb * 64 + kk * 8),
-                                sw128_desc(va + static_cast<uint32_t>(kk * 2048), kTcKVBytes / 2, 1024), id_o,
-                                (j > 0 || kk > 0) ? 1u : 0u);
-                umma_commit(&pvdone[sb]);
-                umma_commit(&vempty[st]);
+                    for (int kk = 0; kk < 4; ++kk)  // 64 keys = 4 steps of 16: P columns kk*8, V key groups 2kk
+                        umma_tmem_a(t_o, t_s + static_cast<uint32_t>(sb * 64 + kk * 8),
+                                    vds + static_cast<uint64_t>((kk * 2048) >> 4), id_o, (j > 0 || kk > 0) ? 1u : 0u);
+                    umma_commit(&pvdone[sb]);
+                    umma_commit(&vempty[st]);
+                }
+                __syncwarp();
             }
             // every MMA issued here is done before the CTA releases TMEM and shared memory
-            umma_commit(&drain);
-            const long long t0 = spin_clock();
-            while (!mbar_try_wait(&drain, 0) && spin_clock() - t0 < kWaitLimitCycles) {
+            if (leader) {
+                umma_commit(&drain);
+                const long long t0 = spin_clock();
+                while (!mbar_try_wait(&drain, 0) && spin_clock() - t0 < kWaitLimitCycles) {
+                }
             }
+            __syncwarp();
         }
     } else {
         // ------------------------------------------------ softmax, output (warps 0..3)
