@@ -101,7 +101,6 @@ __device__ __forceinline__ GemmPlan phase_plan(const ChainPhase& P, int rows) {
         p.total = static_cast<long long>(p.m_tiles) * nt * p.kb;
         const long long min_iters = (p.kb + 29) / 30;  // at most 31 parts per tile, as on the host
         if (p.grid > p.total / min_iters) p.grid = static_cast<int>(p.total / min_iters);
-        if (p.small) p.grid = p.m_tiles * nt;  // a tile each
     }
     return p;
 }
@@ -662,7 +661,7 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
     // TMEM: two accumulators of acc_cols columns, then (token tiles up to 128) the staged old
     // residual of the finisher's tile, x_cols columns
     const uint32_t t_x =
-        !WIDE && ca.x_cols ? tmem_base + static_cast<uint32_t>(ca.x_col0) + (static_cast<uint32_t>(quarter * 32) << 16)
+        !WIDE && ca.x_cols ? tmem_base + static_cast<uint32_t>(2 * ca.acc_cols) + (static_cast<uint32_t>(quarter * 32) << 16)
                   : 0u;
     int rs_nt = -1, ids_nt = -1;
     int prepared = -1;
@@ -764,16 +763,6 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
 #pragma unroll 1
             for (int c = 0; c < nchunks; ++c) {
                 constexpr bool x_ahead = WIDE && EPI == EPI_RESID;
-                if constexpr (!WIDE) {
-                    // (a small plan's k-blocks, each in its accumulator, summed in order)
-                    tmem_ld_32x16(t_acc + static_cast<uint32_t>(half * 16), v);
-                    for (int k = 1; k < (ca.kacc ? p.kb : 1); ++k) {
-                        float w[16];
-                        tmem_ld_32x16(t_acc + static_cast<uint32_t>(32 * k + half * 16), w);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] += w[j];
-                    }
-                }
                 if constexpr (x_ahead) {
                     tmem_ld_32x16(t_acc + static_cast<uint32_t>(c * 32 + half * 16), v);
 #pragma unroll
@@ -783,7 +772,7 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
                 epilogue_c32<EPI, kPass1, WIDE>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
                                                 t_acc + static_cast<uint32_t>(c * 32),
                                                 t_x ? t_x + static_cast<uint32_t>(c * 32) : 0u, esm, e, half, quarter,
-                                                lane, status, x_ahead || !WIDE ? v : nullptr, nullptr, x_ahead, es.buf);
+                                                lane, status, x_ahead ? v : nullptr, nullptr, x_ahead, es.buf);
                 es.buf ^= 1;
             }
         }
@@ -992,7 +981,7 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
             tc_fence_before();
             mbar_arrive(&tempty[es.acc]);
         }
-        if (ca.kacc || ++es.acc == 2) {
+        if (++es.acc == 2) {
             es.acc = 0;
             es.acc_phase ^= 1u;
         }
@@ -1187,80 +1176,73 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
 
     if (warp == 0) {
         // ---------------------------------------------------------- weight producer
-        // The whole warp runs the loop, its slot waits voted warp-wide, so that the copies'
-        // addresses stay warp-uniform values, and one elected lane issues them.
-        const bool leader = elect_one();
-        const int urows = __shfl_sync(0xffffffffu, rows, 0);
-        const uint64_t pol_w = policy_evict_first();
-        const int ring = Q4 ? R : S;
-        int stage = 0, used = 0;  // slots that have held a copy
-        uint32_t par = 0;
-        bool stop = false;
-        constexpr uint32_t tile_bytes = Q4 ? kQ4TileBytes : kABytes;
-        for (int ph = 0; ph < ca.n_phases && !stop; ++ph) {
-            const GemmPlan p = phase_plan(ca.ph[ph], urows);
-            if (static_cast<int>(blockIdx.x) >= p.grid) continue;
-            const int it0 = static_cast<int>(range_begin(blockIdx.x, p.total, p.grid));
-            const int it1 = static_cast<int>(range_begin(blockIdx.x + 1, p.total, p.grid));
-            unsigned long long* tr =
-                (leader && ca.ph[ph].ep.trace) ? ca.ph[ph].ep.trace + static_cast<size_t>(blockIdx.x) * kTrSlots : nullptr;
-            if (tr) tr[kTrStart] = global_ns();
-            // (m-tile, k-block) walked incrementally: no division in the loop
-            int tile = it0 / p.kb, k = it0 - tile * p.kb;
-            int nt = tile / p.m_tiles, mt = tile - nt * p.m_tiles;
-            const char* const w0 = reinterpret_cast<const char*>(ca.ph[ph].w_tiles);
-            const char* wt = w0 + (static_cast<size_t>(mt) * p.kb + k) * tile_bytes;  // tile-major: (mt*kb + k) tiles
-            for (int it = it0; it < it1;) {
-                const int n = (a_tm && k + 1 < p.kb && it + 1 < it1) ? 2 : 1;  // k-blocks of this stage
-                // 4-bit weights: the raw tile goes to its own ring; the dequantizing warps fill the A
-                // stage.  A stages in tensor memory: raw slot s belongs to A stage s, and is free
-                // again once the MMAs that read that stage are done; a pair of tiles of one row
-                // block is one contiguous copy
-                uint64_t* const slot_free = Q4 && !a_tm ? &rempty[stage] : &empty[stage];
-                if (!__all_sync(0xffffffffu, mbar_wait(slot_free, par ^ 1u, s_abort, status))) {
-                    stop = true;
-                    break;
-                }
-                if (leader) {
+        if (lane == 0) {
+            const uint64_t pol_w = policy_evict_first();
+            int stage = 0;
+            uint32_t par = 0;
+            uint32_t pending = 0, pend_par = 0;
+            constexpr uint32_t tile_bytes = Q4 ? kQ4TileBytes : kABytes;
+            for (int ph = 0; ph < ca.n_phases && !*s_abort; ++ph) {
+                const GemmPlan p = phase_plan(ca.ph[ph], rows);
+                if (static_cast<int>(blockIdx.x) >= p.grid) continue;
+                const int it0 = static_cast<int>(range_begin(blockIdx.x, p.total, p.grid));
+                const int it1 = static_cast<int>(range_begin(blockIdx.x + 1, p.total, p.grid));
+                unsigned long long* tr = ca.ph[ph].ep.trace ? ca.ph[ph].ep.trace + static_cast<size_t>(blockIdx.x) * kTrSlots : nullptr;
+                if (tr) tr[kTrStart] = global_ns();
+                // (m-tile, k-block) walked incrementally: no division in the loop
+                int tile = it0 / p.kb, k = it0 - tile * p.kb;
+                int nt = tile / p.m_tiles, mt = tile - nt * p.m_tiles;
+                const char* wt = reinterpret_cast<const char*>(ca.ph[ph].w_tiles);
+                size_t woff = (static_cast<size_t>(mt) * p.kb + k) * tile_bytes;  // tile-major: (mt*kb + k) tiles
+                for (int it = it0; it < it1;) {
+                    const int n = (a_tm && k + 1 < p.kb && it + 1 < it1) ? 2 : 1;  // k-blocks of this stage
                     if constexpr (Q4) {
+                        // the raw tile goes to its own ring; the dequantizing warps fill the A stage.
+                        // A stages in tensor memory: raw slot s belongs to A stage s, and is free
+                        // again once the MMAs that read that stage are done; a pair of tiles of
+                        // one row block is one contiguous copy
+                        if (!mbar_wait(a_tm ? &empty[stage] : &rempty[stage], par ^ 1u, s_abort, status)) break;
                         mbar_arrive_expect_tx(&rfull[stage], n * kQ4TileBytes);
-                        bulk_load_hint(sRaw + static_cast<size_t>(stage) * raw_slot, wt, n * kQ4TileBytes, &rfull[stage],
-                                       pol_w);
+                        bulk_load_hint(sRaw + static_cast<size_t>(stage) * raw_slot, wt + woff, n * kQ4TileBytes,
+                                       &rfull[stage], pol_w);
                     } else {
+                        if (!mbar_wait(&empty[stage], par ^ 1u, s_abort, status)) break;
                         mbar_arrive_expect_tx(&full[stage], kABytes + b_bytes);
-                        if (w0)
-                            bulk_load_hint(sA + static_cast<size_t>(stage) * kABytes, wt, kABytes, &full[stage], pol_w);
+                        if (wt)
+                            bulk_load_hint(sA + static_cast<size_t>(stage) * kABytes, wt + woff, kABytes,
+                                           &full[stage], pol_w);
                         else
                             tma_load_2d(sA + static_cast<size_t>(stage) * kABytes, &maps.w[ph], k * kBK, mt * kBM,
                                         &full[stage], pol_w);
                     }
-                }
-                __syncwarp();
-                used = max(used, stage + 1);
-                if (++stage == ring) {
-                    stage = 0;
-                    par ^= 1u;
-                }
-                it += n;
-                wt += static_cast<size_t>(n) * tile_bytes;
-                k += n;
-                if (k == p.kb) {
-                    k = 0;
-                    if (++mt == p.m_tiles) {
-                        mt = 0;
-                        wt = w0;
+                    pending |= 1u << stage;
+                    pend_par = (pend_par & ~(1u << stage)) | (par << stage);
+                    if (++stage == (Q4 ? R : S)) {
+                        stage = 0;
+                        par ^= 1u;
+                    }
+                    it += n;
+                    woff += static_cast<size_t>(n) * tile_bytes;
+                    k += n;
+                    if (k == p.kb) {
+                        k = 0;
+                        if (++mt == p.m_tiles) {
+                            mt = 0;
+                            woff = 0;
+                            ++nt;
+                        }
                     }
                 }
             }
-        }
-        if (leader && *s_abort) {
-            // let the copies in flight land before the CTA's shared memory is released (a
-            // stage whose operand was never issued does not complete: one deadline for all)
-            const long long t0 = spin_clock();
-            for (int s = 0; s < used; ++s) {
-                uint64_t* bar = Q4 ? &rfull[s] : &full[s];
-                const uint32_t last = s < stage ? par : par ^ 1u;  // the slot's last use
-                while (!mbar_try_wait(bar, last) && spin_clock() - t0 < kWaitLimitCycles) {
+            if (*s_abort) {
+                // let the copies in flight land before the CTA's shared memory is released (a
+                // stage whose operand was never issued does not complete: one deadline for all)
+                const long long t0 = spin_clock();
+                for (int s = 0; s < (Q4 ? R : S); ++s) {
+                    if (!(pending >> s & 1u)) continue;
+                    uint64_t* bar = Q4 ? &rfull[s] : &full[s];
+                    while (!mbar_try_wait(bar, (pend_par >> s) & 1u) && spin_clock() - t0 < kWaitLimitCycles) {
+                    }
                 }
             }
         }
@@ -1277,7 +1259,7 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
         const int urows = __shfl_sync(0xffffffffu, rows, 0);
         int stage = 0;
         uint32_t par = 0;
-        int used = 0;  // slots that have held a copy
+        uint32_t bpend = 0, bpend_par = 0;  // Q4: operand copies issued (for the drain on abort)
         bool stop = false;
         if (ca.gate) {  // the bounded-wait test hook (see ChainArgs::gate)
             int open = 1;
@@ -1297,11 +1279,6 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
             // lane l, bit w = tile 32w + l (a flag, once complete, stays so for the launch)
             uint32_t mine = 0;
             int mine_nt = -1;
-            // and (4-bit weights, where this warp's instructions pace the loop: a step over 32 tokens
-            // 714 -> 689 us; with bf16 weights the stream does) the k-blocks [k_lo, k_hi) known to
-            // be ready from them: the loop looks at the tiles only when it leaves that run
-            const int k_shift = dep_shift - 6;  // k-blocks per producing tile (dep_rows >= 64)
-            int k_lo = 0, k_hi = 0;
             int tile = it0 / p.kb, k = it0 - tile * p.kb;
             int nt = tile / p.m_tiles, mt = tile - nt * p.m_tiles;
             for (int it = it0; it < it1;) {
@@ -1311,13 +1288,11 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                     break;
                 }
                 for (int j = 0; dep && j < n; ++j) {
+                    const int pmt = ((k + j) * kBK) >> dep_shift;
                     if (nt != mine_nt) {
                         mine = 0;
                         mine_nt = nt;
-                        k_lo = k_hi = 0;
                     }
-                    if (Q4 && k + j >= k_lo && k + j < k_hi) continue;
-                    const int pmt = (k + j) >> k_shift;
                     if (!(__shfl_sync(0xffffffffu, mine, pmt & 31) >> (pmt >> 5) & 1u)) {
                         // poll the 32 producing tiles around pmt (one acquire load per lane) until
                         // pmt is complete; what is seen complete is kept for the later k-blocks
@@ -1346,23 +1321,20 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                         }
                         if (stop) break;
                     }
-                    if constexpr (Q4) {  // the run of complete tiles from pmt on, inside its group of 32
-                        const uint32_t open = ~(__ballot_sync(0xffffffffu, mine >> (pmt >> 5) & 1u) >> (pmt & 31));
-                        k_lo = pmt << k_shift;
-                        k_hi = (pmt + (open ? __ffs(open) - 1 : 32)) << k_shift;
-                    }
                 }
                 if (stop) break;
                 if (leader) {
                     uint64_t* fb = Q4 ? &bfull[stage] : &full[stage];
-                    if constexpr (Q4)  // its own barrier; the A part of the stage arrives by the dequantizers
+                    if constexpr (Q4) {  // its own barrier; the A part of the stage arrives by the dequantizers
                         mbar_arrive_expect_tx(fb, n * b_bytes);
+                        bpend |= 1u << stage;
+                        bpend_par = (bpend_par & ~(1u << stage)) | (par << stage);
+                    }
                     for (int j = 0; j < n; ++j)
                         tma_load_2d(sB + static_cast<size_t>(stage) * b_slot + static_cast<size_t>(j) * b_bytes, &maps.x[ph],
                                     (k + j) * kBK, nt * ca.ntile, fb, pol_x);
                 }
                 __syncwarp();
-                used = max(used, stage + 1);
                 if (++stage == SB) {
                     stage = 0;
                     par ^= 1u;
@@ -1383,8 +1355,8 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
             // before the CTA's shared memory is released (one deadline for all)
             if (leader && *s_abort) {
                 const long long t0 = spin_clock();
-                for (int b = 0; b < used; ++b)
-                    while (!mbar_try_wait(&bfull[b], b < stage ? par : par ^ 1u) &&
+                for (int b = 0; b < SB; ++b)
+                    while ((bpend >> b & 1u) && !mbar_try_wait(&bfull[b], (bpend_par >> b) & 1u) &&
                            spin_clock() - t0 < kWaitLimitCycles) {
                     }
             }
@@ -1490,9 +1462,6 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                 const uint32_t d_tmem = tbase + static_cast<uint32_t>(acc * acc_cols);
                 for (int k = k_lo; k < k_hi;) {
                     const int n = (a_tm && k + 1 < k_hi) ? 2 : 1;  // k-blocks of this stage
-                    // a small plan gives every k-block of its tile an accumulator of its own
-                    const uint32_t d_k = d_tmem + (ca.kacc ? static_cast<uint32_t>(32 * k) : 0u);
-                    const uint32_t add = ca.kacc || k == k_lo ? 0u : 1u;  // to what is in it
                     const bool got = mbar_wait(&full[stage], par, s_abort, status) &&
                                      (!Q4 || mbar_wait(&bfull[bstage], bpar, s_abort, status));
                     if (!__all_sync(0xffffffffu, got)) {
@@ -1509,20 +1478,21 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                             const uint32_t a_t = tbase + static_cast<uint32_t>(ca.a_col0 + stage * kBK);
 #pragma unroll
                             for (int kk = 0; kk < kBK / 16; ++kk)
-                                umma_bf16_tmem_a(d_k, a_t + static_cast<uint32_t>(kk * 8), bdesc + 2ull * kk, idesc,
-                                                 kk > 0 ? 1u : add);
+                                umma_bf16_tmem_a(d_tmem, a_t + static_cast<uint32_t>(kk * 8), bdesc + 2ull * kk, idesc,
+                                                 (k > k_lo || kk > 0) ? 1u : 0u);
                             if (n == 2) {
                                 const uint64_t bdesc1 = sw128_kmajor_desc(smem_u32(b_st + b_bytes));
 #pragma unroll
                                 for (int kk = 0; kk < kBK / 16; ++kk)
-                                    umma_bf16_tmem_a(d_k, a_t + static_cast<uint32_t>(32 + kk * 8), bdesc1 + 2ull * kk,
+                                    umma_bf16_tmem_a(d_tmem, a_t + static_cast<uint32_t>(32 + kk * 8), bdesc1 + 2ull * kk,
                                                      idesc, 1u);
                             }
                         } else {
                             const uint64_t adesc = sw128_kmajor_desc(smem_u32(sA + static_cast<size_t>(stage) * kABytes));
 #pragma unroll
                             for (int kk = 0; kk < kBK / 16; ++kk)
-                                umma_bf16(d_k, adesc + 2ull * kk, bdesc + 2ull * kk, idesc, kk > 0 ? 1u : add);
+                                umma_bf16(d_tmem, adesc + 2ull * kk, bdesc + 2ull * kk, idesc,
+                                          (k > k_lo || kk > 0) ? 1u : 0u);
                         }
                         umma_commit(&empty[stage]);
                         if constexpr (Q4) umma_commit(&bempty[bstage]);
@@ -1544,7 +1514,7 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                 if (stop) break;
                 if (leader) umma_commit(&tfull[acc]);
                 __syncwarp();
-                if (ca.kacc || ++acc == 2) {
+                if (++acc == 2) {
                     acc = 0;
                     acc_phase ^= 1u;
                 }
@@ -1589,19 +1559,14 @@ static int pow2ceil(int x) {
     return p;
 }
 
-bool gemm_small(int M, int N, int K, int sms) {
-    const long long n32 = N > 256 ? (N + 31) / 32 : 8;  // one answer for every batch up to 256 tokens
-    return (K + kBK - 1) / kBK <= kSmallKb && ((M + kBM - 1) / kBM) * n32 <= sms;
-}
-
-GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi, bool small) {
+GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi) {
     GemmPlan p{};
     p.M = M;
     p.N = N;
     p.K = K;
-    p.n_tiles = small ? (N + 31) / 32 : (N + 255) / 256;
+    p.n_tiles = (N + 255) / 256;
     const int per = (N + p.n_tiles - 1) / p.n_tiles;
-    p.ntile = small ? 32 : ((per + 31) / 32) * 32;
+    p.ntile = ((per + 31) / 32) * 32;
     p.m_tiles = (M + kBM - 1) / kBM;
     p.kb = (K + kBK - 1) / kBK;
     p.total = static_cast<long long>(p.m_tiles) * p.n_tiles * p.kb;
@@ -1611,8 +1576,6 @@ GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi, bool small) {
     const long long min_iters = (p.kb + 29) / 30;
     if (p.grid > p.total / min_iters) p.grid = static_cast<int>(p.total / min_iters);
     if (p.grid < 1) p.grid = 1;
-    p.small = small ? 1 : 0;
-    if (small) p.grid = p.m_tiles * p.n_tiles;  // a tile each
     p.slots = p.ntile > 32 ? 2 : 1;
     p.pdl = true;
     return p;
@@ -1685,11 +1648,10 @@ bool pdl_enabled() { return g_pdl; }
 bool chain_plan(ChainArgs& ca, int smem_budget) {
     if (ca.n_phases < 1 || ca.n_phases > kMaxPhases) return false;
     const int ntile = ca.ph[0].p.ntile;
-    int grid = 0, kb_max = 0;
+    int grid = 0;
     for (int i = 0; i < ca.n_phases; ++i) {
         const GemmPlan& p = ca.ph[i].p;
-        if (p.ntile != ntile || p.N != ca.ph[0].p.N || p.small != ca.ph[0].p.small) return false;
-        kb_max = kb_max > p.kb ? kb_max : p.kb;
+        if (p.ntile != ntile || p.N != ca.ph[0].p.N) return false;
         grid = grid > p.grid ? grid : p.grid;
     }
     for (int i = 1; i < ca.n_phases; ++i)
@@ -1697,16 +1659,12 @@ bool chain_plan(ChainArgs& ca, int smem_budget) {
     const bool c32 = ntile == 32;
     // wider token tiles are tensor-bound: the deepest ring (the attention CTAs' room matters
     // only to the batch-1 weight stream)
-    ca.kacc = ca.ph[0].p.small;
-    if (ca.kacc && kb_max > kSmallKb) return false;
-    // (a small plan takes up to all of tensor memory, so no CTA that wants some may join its own)
-    if (!c32 || ca.kacc) smem_budget = kFullSmem;
+    if (!c32) smem_budget = kFullSmem;
     ca.grid = grid;
     ca.ntile = ntile;
-    ca.acc_cols = ca.kacc ? 32 * kb_max : (c32 ? 32 : pow2ceil(ntile));
+    ca.acc_cols = c32 ? 32 : pow2ceil(ntile);
     ca.x_cols = c32 ? ntile : 0;  // staged old residual (wider tiles read it with the parts)
-    ca.x_col0 = (ca.kacc ? 1 : 2) * ca.acc_cols;
-    ca.tmem_cols = pow2ceil(ca.x_col0 + ca.x_cols);
+    ca.tmem_cols = pow2ceil(2 * ca.acc_cols + ca.x_cols);
     const int stage_bytes = static_cast<int>(kABytes) + ntile * kBK * 2;
     const int fixed0 = 1024 + kTailFloats * 4 + (c32 ? 1 : 2) * kStgBytes + 5 * 8 + 16;
     if (ca.q4) {
@@ -1716,12 +1674,12 @@ bool chain_plan(ChainArgs& ca, int smem_budget) {
         // what is left allows (2 .. 24)
         const int kRaw[3] = {12, 8, 6}, kA[3] = {4, 3, 2};
         const int b_stage = ntile * kBK * 2 + 16;
-        const int a_col0 = ca.x_col0 + ca.x_cols;
+        const int a_col0 = 2 * ca.acc_cols + ca.x_cols;
         // A stages in tensor memory where it holds at least 4 stages of two k-blocks (64 columns
         // each): then raw slots (two tiles each) and A stages are one ring of up to 6 stages, and
         // the operand ring holds up to 12 stages of two k-blocks
         const int tm_stages = (512 - a_col0) / kBK;
-        ca.a_tmem = tm_stages >= 4 && !ca.kacc ? 1 : 0;
+        ca.a_tmem = tm_stages >= 4 ? 1 : 0;
         ca.a_col0 = ca.a_tmem ? a_col0 : 0;
         if (ca.a_tmem) {
             const int n = tm_stages < 6 ? tm_stages : 6;
