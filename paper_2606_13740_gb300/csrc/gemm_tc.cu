@@ -1259,7 +1259,7 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
         const int urows = __shfl_sync(0xffffffffu, rows, 0);
         int stage = 0;
         uint32_t par = 0;
-        uint32_t bpend = 0, bpend_par = 0;  // Q4: operand copies issued (for the drain on abort)
+        int used = 0;  // slots that have held a copy
         bool stop = false;
         if (ca.gate) {  // the bounded-wait test hook (see ChainArgs::gate)
             int open = 1;
@@ -1279,6 +1279,11 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
             // lane l, bit w = tile 32w + l (a flag, once complete, stays so for the launch)
             uint32_t mine = 0;
             int mine_nt = -1;
+            // and (4-bit weights, where this warp's instructions pace the loop: a step over 32 tokens
+            // 714 -> 689 us; with bf16 weights the stream does) the k-blocks [k_lo, k_hi) known to
+            // be ready from them: the loop looks at the tiles only when it leaves that run
+            const int k_shift = dep_shift - 6;  // k-blocks per producing tile (dep_rows >= 64)
+            int k_lo = 0, k_hi = 0;
             int tile = it0 / p.kb, k = it0 - tile * p.kb;
             int nt = tile / p.m_tiles, mt = tile - nt * p.m_tiles;
             for (int it = it0; it < it1;) {
@@ -1288,11 +1293,13 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                     break;
                 }
                 for (int j = 0; dep && j < n; ++j) {
-                    const int pmt = ((k + j) * kBK) >> dep_shift;
                     if (nt != mine_nt) {
                         mine = 0;
                         mine_nt = nt;
+                        k_lo = k_hi = 0;
                     }
+                    if (Q4 && k + j >= k_lo && k + j < k_hi) continue;
+                    const int pmt = (k + j) >> k_shift;
                     if (!(__shfl_sync(0xffffffffu, mine, pmt & 31) >> (pmt >> 5) & 1u)) {
                         // poll the 32 producing tiles around pmt (one acquire load per lane) until
                         // pmt is complete; what is seen complete is kept for the later k-blocks
@@ -1321,20 +1328,23 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                         }
                         if (stop) break;
                     }
+                    if constexpr (Q4) {  // the run of complete tiles from pmt on, inside its group of 32
+                        const uint32_t open = ~(__ballot_sync(0xffffffffu, mine >> (pmt >> 5) & 1u) >> (pmt & 31));
+                        k_lo = pmt << k_shift;
+                        k_hi = (pmt + (open ? __ffs(open) - 1 : 32)) << k_shift;
+                    }
                 }
                 if (stop) break;
                 if (leader) {
                     uint64_t* fb = Q4 ? &bfull[stage] : &full[stage];
-                    if constexpr (Q4) {  // its own barrier; the A part of the stage arrives by the dequantizers
+                    if constexpr (Q4)  // its own barrier; the A part of the stage arrives by the dequantizers
                         mbar_arrive_expect_tx(fb, n * b_bytes);
-                        bpend |= 1u << stage;
-                        bpend_par = (bpend_par & ~(1u << stage)) | (par << stage);
-                    }
                     for (int j = 0; j < n; ++j)
                         tma_load_2d(sB + static_cast<size_t>(stage) * b_slot + static_cast<size_t>(j) * b_bytes, &maps.x[ph],
                                     (k + j) * kBK, nt * ca.ntile, fb, pol_x);
                 }
                 __syncwarp();
+                used = max(used, stage + 1);
                 if (++stage == SB) {
                     stage = 0;
                     par ^= 1u;
@@ -1355,8 +1365,8 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
             // before the CTA's shared memory is released (one deadline for all)
             if (leader && *s_abort) {
                 const long long t0 = spin_clock();
-                for (int b = 0; b < SB; ++b)
-                    while ((bpend >> b & 1u) && !mbar_try_wait(&bfull[b], (bpend_par >> b) & 1u) &&
+                for (int b = 0; b < used; ++b)
+                    while (!mbar_try_wait(&bfull[b], b < stage ? par : par ^ 1u) &&
                            spin_clock() - t0 < kWaitLimitCycles) {
                     }
             }
