@@ -1176,73 +1176,80 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
 
     if (warp == 0) {
         // ---------------------------------------------------------- weight producer
-        if (lane == 0) {
-            const uint64_t pol_w = policy_evict_first();
-            int stage = 0;
-            uint32_t par = 0;
-            uint32_t pending = 0, pend_par = 0;
-            constexpr uint32_t tile_bytes = Q4 ? kQ4TileBytes : kABytes;
-            for (int ph = 0; ph < ca.n_phases && !*s_abort; ++ph) {
-                const GemmPlan p = phase_plan(ca.ph[ph], rows);
-                if (static_cast<int>(blockIdx.x) >= p.grid) continue;
-                const int it0 = static_cast<int>(range_begin(blockIdx.x, p.total, p.grid));
-                const int it1 = static_cast<int>(range_begin(blockIdx.x + 1, p.total, p.grid));
-                unsigned long long* tr = ca.ph[ph].ep.trace ? ca.ph[ph].ep.trace + static_cast<size_t>(blockIdx.x) * kTrSlots : nullptr;
-                if (tr) tr[kTrStart] = global_ns();
-                // (m-tile, k-block) walked incrementally: no division in the loop
-                int tile = it0 / p.kb, k = it0 - tile * p.kb;
-                int nt = tile / p.m_tiles, mt = tile - nt * p.m_tiles;
-                const char* wt = reinterpret_cast<const char*>(ca.ph[ph].w_tiles);
-                size_t woff = (static_cast<size_t>(mt) * p.kb + k) * tile_bytes;  // tile-major: (mt*kb + k) tiles
-                for (int it = it0; it < it1;) {
-                    const int n = (a_tm && k + 1 < p.kb && it + 1 < it1) ? 2 : 1;  // k-blocks of this stage
+        // The whole warp runs the loop, its slot waits voted warp-wide, so that the copies'
+        // addresses stay warp-uniform values, and one elected lane issues them.
+        const bool leader = elect_one();
+        const int urows = __shfl_sync(0xffffffffu, rows, 0);
+        const uint64_t pol_w = policy_evict_first();
+        const int ring = Q4 ? R : S;
+        int stage = 0, used = 0;  // slots that have held a copy
+        uint32_t par = 0;
+        bool stop = false;
+        constexpr uint32_t tile_bytes = Q4 ? kQ4TileBytes : kABytes;
+        for (int ph = 0; ph < ca.n_phases && !stop; ++ph) {
+            const GemmPlan p = phase_plan(ca.ph[ph], urows);
+            if (static_cast<int>(blockIdx.x) >= p.grid) continue;
+            const int it0 = static_cast<int>(range_begin(blockIdx.x, p.total, p.grid));
+            const int it1 = static_cast<int>(range_begin(blockIdx.x + 1, p.total, p.grid));
+            unsigned long long* tr =
+                (leader && ca.ph[ph].ep.trace) ? ca.ph[ph].ep.trace + static_cast<size_t>(blockIdx.x) * kTrSlots : nullptr;
+            if (tr) tr[kTrStart] = global_ns();
+            // (m-tile, k-block) walked incrementally: no division in the loop
+            int tile = it0 / p.kb, k = it0 - tile * p.kb;
+            int nt = tile / p.m_tiles, mt = tile - nt * p.m_tiles;
+            const char* const w0 = reinterpret_cast<const char*>(ca.ph[ph].w_tiles);
+            const char* wt = w0 + (static_cast<size_t>(mt) * p.kb + k) * tile_bytes;  // tile-major: (mt*kb + k) tiles
+            for (int it = it0; it < it1;) {
+                const int n = (a_tm && k + 1 < p.kb && it + 1 < it1) ? 2 : 1;  // k-blocks of this stage
+                // 4-bit weights: the raw tile goes to its own ring; the dequantizing warps fill the A
+                // stage.  A stages in tensor memory: raw slot s belongs to A stage s, and is free
+                // again once the MMAs that read that stage are done; a pair of tiles of one row
+                // block is one contiguous copy
+                uint64_t* const slot_free = Q4 && !a_tm ? &rempty[stage] : &empty[stage];
+                if (!__all_sync(0xffffffffu, mbar_wait(slot_free, par ^ 1u, s_abort, status))) {
+                    stop = true;
+                    break;
+                }
+                if (leader) {
                     if constexpr (Q4) {
-                        // the raw tile goes to its own ring; the dequantizing warps fill the A stage.
-                        // A stages in tensor memory: raw slot s belongs to A stage s, and is free
-                        // again once the MMAs that read that stage are done; a pair of tiles of
-                        // one row block is one contiguous copy
-                        if (!mbar_wait(a_tm ? &empty[stage] : &rempty[stage], par ^ 1u, s_abort, status)) break;
                         mbar_arrive_expect_tx(&rfull[stage], n * kQ4TileBytes);
-                        bulk_load_hint(sRaw + static_cast<size_t>(stage) * raw_slot, wt + woff, n * kQ4TileBytes,
-                                       &rfull[stage], pol_w);
+                        bulk_load_hint(sRaw + static_cast<size_t>(stage) * raw_slot, wt, n * kQ4TileBytes, &rfull[stage],
+                                       pol_w);
                     } else {
-                        if (!mbar_wait(&empty[stage], par ^ 1u, s_abort, status)) break;
                         mbar_arrive_expect_tx(&full[stage], kABytes + b_bytes);
-                        if (wt)
-                            bulk_load_hint(sA + static_cast<size_t>(stage) * kABytes, wt + woff, kABytes,
-                                           &full[stage], pol_w);
+                        if (w0)
+                            bulk_load_hint(sA + static_cast<size_t>(stage) * kABytes, wt, kABytes, &full[stage], pol_w);
                         else
                             tma_load_2d(sA + static_cast<size_t>(stage) * kABytes, &maps.w[ph], k * kBK, mt * kBM,
                                         &full[stage], pol_w);
                     }
-                    pending |= 1u << stage;
-                    pend_par = (pend_par & ~(1u << stage)) | (par << stage);
-                    if (++stage == (Q4 ? R : S)) {
-                        stage = 0;
-                        par ^= 1u;
-                    }
-                    it += n;
-                    woff += static_cast<size_t>(n) * tile_bytes;
-                    k += n;
-                    if (k == p.kb) {
-                        k = 0;
-                        if (++mt == p.m_tiles) {
-                            mt = 0;
-                            woff = 0;
-                            ++nt;
-                        }
+                }
+                __syncwarp();
+                used = max(used, stage + 1);
+                if (++stage == ring) {
+                    stage = 0;
+                    par ^= 1u;
+                }
+                it += n;
+                wt += static_cast<size_t>(n) * tile_bytes;
+                k += n;
+                if (k == p.kb) {
+                    k = 0;
+                    if (++mt == p.m_tiles) {
+                        mt = 0;
+                        wt = w0;
                     }
                 }
             }
-            if (*s_abort) {
-                // let the copies in flight land before the CTA's shared memory is released (a
-                // stage whose operand was never issued does not complete: one deadline for all)
-                const long long t0 = spin_clock();
-                for (int s = 0; s < (Q4 ? R : S); ++s) {
-                    if (!(pending >> s & 1u)) continue;
-                    uint64_t* bar = Q4 ? &rfull[s] : &full[s];
-                    while (!mbar_try_wait(bar, (pend_par >> s) & 1u) && spin_clock() - t0 < kWaitLimitCycles) {
-                    }
+        }
+        if (leader && *s_abort) {
+            // let the copies in flight land before the CTA's shared memory is released (a
+            // stage whose operand was never issued does not complete: one deadline for all)
+            const long long t0 = spin_clock();
+            for (int s = 0; s < used; ++s) {
+                uint64_t* bar = Q4 ? &rfull[s] : &full[s];
+                const uint32_t last = s < stage ? par : par ^ 1u;  // the slot's last use
+                while (!mbar_try_wait(bar, last) && spin_clock() - t0 < kWaitLimitCycles) {
                 }
             }
         }
