@@ -108,7 +108,8 @@ Layout make_layout(const dllm_config& c) {
     L.part_floats = static_cast<size_t>(kMaxSMs) * (nt_max > 32 ? 2 : 1) * nt_max * 128;
     L.off_part = take(L.part_floats * 4 * kMaxPhases);
     const int mt_max = std::max(std::max(L.head_tiles, L.gu_rows / 128), std::max(L.qkv_rows, L.d_rows) / 128);
-    L.done_len = mt_max * ((L.max_tok + 255) / 256 + 1);
+    // a small plan (32-token tiles) has at most one tile per SM
+    L.done_len = std::max(mt_max * ((L.max_tok + 255) / 256 + 1), kMaxSMs);
     L.cnt_len = L.done_len * 32;
     L.off_cnt = take(static_cast<size_t>(L.cnt_len) * 4 * kMaxPhases);
     L.off_done = take(static_cast<size_t>(L.done_len) * 4 * kMaxPhases * 2);  // done, then done2 slots
@@ -318,11 +319,16 @@ static int forward(dllm_ctx* ctx, int B, int Tw, bool head, int R = 0, bool sls 
     CK(launch_embed(ctx->tok, c.max_ctx, ctx->seq_kv, ctx->emb, ctx->x, ctx->xn, ctx->sq, ctx->cur, ctx->epoch, B, T,
                     d, s, Tw, ctx->trk));
     mark(ctx, DLLM_K_EMBED);
-    const GemmPlan pq = gemm_plan(L.qkv_rows, N, d, ctx->sms, EPI_QKV);
-    const GemmPlan po = gemm_plan(L.o_rows, N, qd, ctx->sms, EPI_RESID);
-    const GemmPlan pg = gemm_plan(L.gu_rows, N, d, ctx->sms, EPI_SWIGLU);
-    const GemmPlan pd = gemm_plan(L.d_rows, N, F, ctx->sms, EPI_RESID);
-    const GemmPlan ph = gemm_plan(L.head_rows, N, d, ctx->sms, EPI_LMHEAD);
+    // the phases of a chain share one token tiling: small only where every layer phase is (and the
+    // head, when it ends the last chain), so that a sequence's sums do not depend on its batch
+    const bool small = gemm_small(L.qkv_rows, N, d, ctx->sms) && gemm_small(L.o_rows, N, qd, ctx->sms) &&
+                       gemm_small(L.gu_rows, N, d, ctx->sms) && gemm_small(L.d_rows, N, F, ctx->sms) &&
+                       gemm_small(L.head_rows, N, d, ctx->sms);
+    const GemmPlan pq = gemm_plan(L.qkv_rows, N, d, ctx->sms, EPI_QKV, small);
+    const GemmPlan po = gemm_plan(L.o_rows, N, qd, ctx->sms, EPI_RESID, small);
+    const GemmPlan pg = gemm_plan(L.gu_rows, N, d, ctx->sms, EPI_SWIGLU, small);
+    const GemmPlan pd = gemm_plan(L.d_rows, N, F, ctx->sms, EPI_RESID, small);
+    const GemmPlan ph = gemm_plan(L.head_rows, N, d, ctx->sms, EPI_LMHEAD, small);
     CUtensorMap tx_xn, tx_attn, tx_h, tx_c;
     if (!make_tmap_bf16(&tx_xn, ctx->xn, N, d, pq.ntile) || !make_tmap_bf16(&tx_attn, ctx->attn, N, qd, po.ntile) ||
         !make_tmap_bf16(&tx_h, ctx->h, N, F, pd.ntile) || !make_tmap_bf16(&tx_c, ctx->sls_x, N, d, ph.ntile))

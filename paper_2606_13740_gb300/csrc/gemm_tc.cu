@@ -101,6 +101,7 @@ __device__ __forceinline__ GemmPlan phase_plan(const ChainPhase& P, int rows) {
         p.total = static_cast<long long>(p.m_tiles) * nt * p.kb;
         const long long min_iters = (p.kb + 29) / 30;  // at most 31 parts per tile, as on the host
         if (p.grid > p.total / min_iters) p.grid = static_cast<int>(p.total / min_iters);
+        if (p.small) p.grid = p.m_tiles * nt;  // a tile each
     }
     return p;
 }
@@ -661,7 +662,7 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
     // TMEM: two accumulators of acc_cols columns, then (token tiles up to 128) the staged old
     // residual of the finisher's tile, x_cols columns
     const uint32_t t_x =
-        !WIDE && ca.x_cols ? tmem_base + static_cast<uint32_t>(2 * ca.acc_cols) + (static_cast<uint32_t>(quarter * 32) << 16)
+        !WIDE && ca.x_cols ? tmem_base + static_cast<uint32_t>(ca.x_col0) + (static_cast<uint32_t>(quarter * 32) << 16)
                   : 0u;
     int rs_nt = -1, ids_nt = -1;
     int prepared = -1;
@@ -763,6 +764,16 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
 #pragma unroll 1
             for (int c = 0; c < nchunks; ++c) {
                 constexpr bool x_ahead = WIDE && EPI == EPI_RESID;
+                if constexpr (!WIDE) {
+                    // (a small plan's k-blocks, each in its accumulator, summed in order)
+                    tmem_ld_32x16(t_acc + static_cast<uint32_t>(half * 16), v);
+                    for (int k = 1; k < (ca.kacc ? p.kb : 1); ++k) {
+                        float w[16];
+                        tmem_ld_32x16(t_acc + static_cast<uint32_t>(32 * k + half * 16), w);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) v[j] += w[j];
+                    }
+                }
                 if constexpr (x_ahead) {
                     tmem_ld_32x16(t_acc + static_cast<uint32_t>(c * 32 + half * 16), v);
 #pragma unroll
@@ -772,7 +783,7 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
                 epilogue_c32<EPI, kPass1, WIDE>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
                                                 t_acc + static_cast<uint32_t>(c * 32),
                                                 t_x ? t_x + static_cast<uint32_t>(c * 32) : 0u, esm, e, half, quarter,
-                                                lane, status, x_ahead ? v : nullptr, nullptr, x_ahead, es.buf);
+                                                lane, status, x_ahead || !WIDE ? v : nullptr, nullptr, x_ahead, es.buf);
                 es.buf ^= 1;
             }
         }
@@ -981,7 +992,7 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
             tc_fence_before();
             mbar_arrive(&tempty[es.acc]);
         }
-        if (++es.acc == 2) {
+        if (ca.kacc || ++es.acc == 2) {
             es.acc = 0;
             es.acc_phase ^= 1u;
         }
@@ -1479,6 +1490,9 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                 const uint32_t d_tmem = tbase + static_cast<uint32_t>(acc * acc_cols);
                 for (int k = k_lo; k < k_hi;) {
                     const int n = (a_tm && k + 1 < k_hi) ? 2 : 1;  // k-blocks of this stage
+                    // a small plan gives every k-block of its tile an accumulator of its own
+                    const uint32_t d_k = d_tmem + (ca.kacc ? static_cast<uint32_t>(32 * k) : 0u);
+                    const uint32_t add = ca.kacc || k == k_lo ? 0u : 1u;  // to what is in it
                     const bool got = mbar_wait(&full[stage], par, s_abort, status) &&
                                      (!Q4 || mbar_wait(&bfull[bstage], bpar, s_abort, status));
                     if (!__all_sync(0xffffffffu, got)) {
@@ -1495,21 +1509,20 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                             const uint32_t a_t = tbase + static_cast<uint32_t>(ca.a_col0 + stage * kBK);
 #pragma unroll
                             for (int kk = 0; kk < kBK / 16; ++kk)
-                                umma_bf16_tmem_a(d_tmem, a_t + static_cast<uint32_t>(kk * 8), bdesc + 2ull * kk, idesc,
-                                                 (k > k_lo || kk > 0) ? 1u : 0u);
+                                umma_bf16_tmem_a(d_k, a_t + static_cast<uint32_t>(kk * 8), bdesc + 2ull * kk, idesc,
+                                                 kk > 0 ? 1u : add);
                             if (n == 2) {
                                 const uint64_t bdesc1 = sw128_kmajor_desc(smem_u32(b_st + b_bytes));
 #pragma unroll
                                 for (int kk = 0; kk < kBK / 16; ++kk)
-                                    umma_bf16_tmem_a(d_tmem, a_t + static_cast<uint32_t>(32 + kk * 8), bdesc1 + 2ull * kk,
+                                    umma_bf16_tmem_a(d_k, a_t + static_cast<uint32_t>(32 + kk * 8), bdesc1 + 2ull * kk,
                                                      idesc, 1u);
                             }
                         } else {
                             const uint64_t adesc = sw128_kmajor_desc(smem_u32(sA + static_cast<size_t>(stage) * kABytes));
 #pragma unroll
                             for (int kk = 0; kk < kBK / 16; ++kk)
-                                umma_bf16(d_tmem, adesc + 2ull * kk, bdesc + 2ull * kk, idesc,
-                                          (k > k_lo || kk > 0) ? 1u : 0u);
+                                umma_bf16(d_k, adesc + 2ull * kk, bdesc + 2ull * kk, idesc, kk > 0 ? 1u : add);
                         }
                         umma_commit(&empty[stage]);
                         if constexpr (Q4) umma_commit(&bempty[bstage]);
@@ -1531,7 +1544,7 @@ __global__ void __launch_bounds__(Q4 ? kChainThreadsQ4 : kChainThreads, 1)
                 if (stop) break;
                 if (leader) umma_commit(&tfull[acc]);
                 __syncwarp();
-                if (++acc == 2) {
+                if (ca.kacc || ++acc == 2) {
                     acc = 0;
                     acc_phase ^= 1u;
                 }
@@ -1576,14 +1589,19 @@ static int pow2ceil(int x) {
     return p;
 }
 
-GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi) {
+bool gemm_small(int M, int N, int K, int sms) {
+    const long long n32 = N > 256 ? (N + 31) / 32 : 8;  // one answer for every batch up to 256 tokens
+    return (K + kBK - 1) / kBK <= kSmallKb && ((M + kBM - 1) / kBM) * n32 <= sms;
+}
+
+GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi, bool small) {
     GemmPlan p{};
     p.M = M;
     p.N = N;
     p.K = K;
-    p.n_tiles = (N + 255) / 256;
+    p.n_tiles = small ? (N + 31) / 32 : (N + 255) / 256;
     const int per = (N + p.n_tiles - 1) / p.n_tiles;
-    p.ntile = ((per + 31) / 32) * 32;
+    p.ntile = small ? 32 : ((per + 31) / 32) * 32;
     p.m_tiles = (M + kBM - 1) / kBM;
     p.kb = (K + kBK - 1) / kBK;
     p.total = static_cast<long long>(p.m_tiles) * p.n_tiles * p.kb;
@@ -1593,6 +1611,8 @@ GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi) {
     const long long min_iters = (p.kb + 29) / 30;
     if (p.grid > p.total / min_iters) p.grid = static_cast<int>(p.total / min_iters);
     if (p.grid < 1) p.grid = 1;
+    p.small = small ? 1 : 0;
+    if (small) p.grid = p.m_tiles * p.n_tiles;  // a tile each
     p.slots = p.ntile > 32 ? 2 : 1;
     p.pdl = true;
     return p;
@@ -1665,10 +1685,11 @@ bool pdl_enabled() { return g_pdl; }
 bool chain_plan(ChainArgs& ca, int smem_budget) {
     if (ca.n_phases < 1 || ca.n_phases > kMaxPhases) return false;
     const int ntile = ca.ph[0].p.ntile;
-    int grid = 0;
+    int grid = 0, kb_max = 0;
     for (int i = 0; i < ca.n_phases; ++i) {
         const GemmPlan& p = ca.ph[i].p;
-        if (p.ntile != ntile || p.N != ca.ph[0].p.N) return false;
+        if (p.ntile != ntile || p.N != ca.ph[0].p.N || p.small != ca.ph[0].p.small) return false;
+        kb_max = kb_max > p.kb ? kb_max : p.kb;
         grid = grid > p.grid ? grid : p.grid;
     }
     for (int i = 1; i < ca.n_phases; ++i)
@@ -1676,12 +1697,16 @@ bool chain_plan(ChainArgs& ca, int smem_budget) {
     const bool c32 = ntile == 32;
     // wider token tiles are tensor-bound: the deepest ring (the attention CTAs' room matters
     // only to the batch-1 weight stream)
-    if (!c32) smem_budget = kFullSmem;
+    ca.kacc = ca.ph[0].p.small;
+    if (ca.kacc && kb_max > kSmallKb) return false;
+    // (a small plan takes up to all of tensor memory, so no CTA that wants some may join its own)
+    if (!c32 || ca.kacc) smem_budget = kFullSmem;
     ca.grid = grid;
     ca.ntile = ntile;
-    ca.acc_cols = c32 ? 32 : pow2ceil(ntile);
+    ca.acc_cols = ca.kacc ? 32 * kb_max : (c32 ? 32 : pow2ceil(ntile));
     ca.x_cols = c32 ? ntile : 0;  // staged old residual (wider tiles read it with the parts)
-    ca.tmem_cols = pow2ceil(2 * ca.acc_cols + ca.x_cols);
+    ca.x_col0 = (ca.kacc ? 1 : 2) * ca.acc_cols;
+    ca.tmem_cols = pow2ceil(ca.x_col0 + ca.x_cols);
     const int stage_bytes = static_cast<int>(kABytes) + ntile * kBK * 2;
     const int fixed0 = 1024 + kTailFloats * 4 + (c32 ? 1 : 2) * kStgBytes + 5 * 8 + 16;
     if (ca.q4) {
@@ -1691,12 +1716,12 @@ bool chain_plan(ChainArgs& ca, int smem_budget) {
         // what is left allows (2 .. 24)
         const int kRaw[3] = {12, 8, 6}, kA[3] = {4, 3, 2};
         const int b_stage = ntile * kBK * 2 + 16;
-        const int a_col0 = 2 * ca.acc_cols + ca.x_cols;
+        const int a_col0 = ca.x_col0 + ca.x_cols;
         // A stages in tensor memory where it holds at least 4 stages of two k-blocks (64 columns
         // each): then raw slots (two tiles each) and A stages are one ring of up to 6 stages, and
         // the operand ring holds up to 12 stages of two k-blocks
         const int tm_stages = (512 - a_col0) / kBK;
-        ca.a_tmem = tm_stages >= 4 ? 1 : 0;
+        ca.a_tmem = tm_stages >= 4 && !ca.kacc ? 1 : 0;
         ca.a_col0 = ca.a_tmem ? a_col0 : 0;
         if (ca.a_tmem) {
             const int n = tm_stages < 6 ? tm_stages : 6;

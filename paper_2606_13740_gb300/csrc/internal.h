@@ -94,6 +94,7 @@ struct GemmPlan {
     int m_tiles, n_tiles, kb;
     long long total;     // m_tiles * n_tiles * kb iterations of 64-wide K blocks
     int grid;            // CTAs (stream-K partition of the iterations)
+    int small;           // whole 32-token tiles, one per CTA (gemm_plan)
     int slots;           // split partials a CTA may store: two let a wide tile's parts share its epilogue
     bool pdl;            // launch with programmatic dependent launch (the step's chain)
 };
@@ -132,7 +133,8 @@ struct ChainPhase {
 struct ChainArgs {
     int n_phases;
     int grid, stages, ntile, acc_cols, tmem_cols;
-    int x_cols;          // TMEM columns for the staged old residual (0: none)
+    int x_cols, x_col0;  // TMEM columns for the staged old residual (0: none) and the first of them
+    int kacc;            // small plans: one set of accumulators, 32 columns for each k-block of a tile
     size_t smem;
     const int* epoch;    // device step counter; tag = *epoch * tag_mul + tag_add (null: tag = tag_add)
     int tag_mul, tag_add;
@@ -171,7 +173,15 @@ cudaError_t chain_init_attrs();
 
 // Tiling of one projection: token tiles of at most 256 (multiples of 32), 128 weight rows
 // per tile, 64-wide k-blocks, grid = min(iterations, grid_max).
-GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi);
+// small: whole tiles of 32 tokens, one per CTA.  For projections of few k-blocks and no more such
+// tiles than SMs (gemm_small) a tile's k-blocks take a CTA less than the exchange of its parts
+// would, 3 to 4 us a phase.  Every k-block has an accumulator of its own and the epilogue sums them
+// in order, so the sums are those of one k-block per CTA bit for bit, whatever the batch.  The
+// 256-wide two-layer model's step: 32 tokens 135 -> 106 us, 8 x 32 tokens 208 -> 120 us.  kSmallKb: the accumulators
+// of 32 columns that fit tensor memory beside the old residual.
+constexpr int kSmallKb = 15;
+bool gemm_small(int M, int N, int K, int sms);
+GemmPlan gemm_plan(int M, int N, int K, int grid_max, int epi, bool small = false);
 // Split-partial floats a single-projection launch of plan p needs (ntile x 128 per slot);
 // gemm_launch rejects a smaller Scratch.
 inline size_t gemm_partial_floats(const GemmPlan& p) {

@@ -128,7 +128,8 @@ static int gemm_impl(const void* W, const void* X, float* D, int M, int N, int K
     int sms = sm_count();
     if (sms <= 0) return op_fail(DLLM_ECUDA, "no CUDA device");
     if (gemm_init_attrs() != cudaSuccess) return op_fail(DLLM_ECUDA, "attribute setup failed");
-    GemmPlan p = gemm_plan(M, N, K, (grid > 0 && grid < sms) ? grid : sms, EPI_F32);
+    // a grid that the caller chose is kept
+    GemmPlan p = gemm_plan(M, N, K, (grid > 0 && grid < sms) ? grid : sms, EPI_F32, grid <= 0 && gemm_small(M, N, K, sms));
     p.pdl = false;  // the operands come from the caller's kernels
     CUtensorMap tw, tx;
     if (!make_tmap_bf16(&tw, W, M, K, 128) || !make_tmap_bf16(&tx, X, N, K, p.ntile))
@@ -234,7 +235,7 @@ int dllm_op_lmhead(const void* W, const void* X, const int32_t* cur, int32_t* x0
     int sms = sm_count();
     if (sms <= 0) return op_fail(DLLM_ECUDA, "no CUDA device");
     if (gemm_init_attrs() != cudaSuccess) return op_fail(DLLM_ECUDA, "attribute setup failed");
-    GemmPlan p = gemm_plan(V, N, d, sms, EPI_LMHEAD);
+    GemmPlan p = gemm_plan(V, N, d, sms, EPI_LMHEAD, gemm_small(V, N, d, sms));
     p.pdl = false;
     CUtensorMap tw, tx;
     if (!make_tmap_bf16(&tw, W, V, d, 128) || !make_tmap_bf16(&tx, X, N, d, p.ntile))

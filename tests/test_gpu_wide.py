@@ -42,6 +42,21 @@ def test_wide_split_tiles(pkg, M, N, K, grid):
     assert torch.equal(D, pkg.dllm_op_gemm(W, X, M, N, K, grid=grid))
 
 
+# the last sizes whose tiles run whole, 32 tokens and one CTA each (up to 960 columns deep, at most
+# one tile per SM), and the first past them
+@pytest.mark.parametrize("M,N,K", [
+    (768, 33, 256), (128, 1, 8), (2432, 256, 960), (2433, 256, 960), (2432, 250, 968), (256, 2432, 688),
+    (256, 2433, 688), (128, 4096, 64), (130, 31, 960), (130, 31, 968),
+])
+def test_small_whole_tiles(pkg, M, N, K):
+    g = torch.Generator().manual_seed(M + N + K)
+    W, X = _bf16(g, M, K, sigma=0.05), _bf16(g, N, K)
+    D = pkg.dllm_op_gemm(W, X, M, N, K)
+    w, x = W.double(), X.double()
+    tol = 1e-5 * x.norm(dim=1)[:, None] * w.norm(dim=1)[None, :]  # as above
+    assert bool(((D.double() - x @ w.T).abs() <= tol).all())
+
+
 @pytest.mark.parametrize("V,N,d", [(1024, 251, 4096), (512, 96, 2048), (4096, 64, 512)])
 def test_wide_head_split_tiles(pkg, V, N, d):
     g = torch.Generator().manual_seed(V + N)
