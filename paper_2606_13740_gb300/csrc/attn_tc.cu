@@ -550,11 +550,22 @@ AttnPlan attn_plan_tc(int B, int T, int H, int Hkv, int max_keys, int sms) {
     a.qtiles = (H / Hkv * T + kTcRows - 1) / kTcRows;
     const int units = B * Hkv * a.qtiles;
     const int blocks = (max_keys + kTcKeys - 1) / kTcKeys;
-    // key splits (cluster size): about two CTAs per SM, at most one split per sub-block
-    int c = (2 * sms + units - 1) / units;
-    if (c > kTcMaxCluster) c = kTcMaxCluster;
-    if (c > blocks) c = blocks;
-    if (c < 1) c = 1;
+    // Key splits (cluster size).  Units that fill two CTAs per SM by themselves run whole: a last
+    // wave of few CTAs runs faster than a full one, and splits cost a merge (332 units of 24
+    // sub-blocks in two splits: 100 -> 121 us).  Otherwise the split whose waves take the fewest
+    // sub-blocks, a wave costing about kWaveBlocks more for its start, merge and end, the smaller
+    // of equals: a few CTAs past a wave cost a second one (6 x 96 tokens of 28 heads over 4, 144
+    // units: three splits 80 us a call, two 68 us; 5 x 32 tokens, 40 units: eight 80 us, six 70 us).
+    constexpr int kWaveBlocks = 4;
+    const int wave = 2 * sms;
+    int c = 1, best = 0;
+    for (int k = 1; units < wave && k <= kTcMaxCluster && k <= blocks; ++k) {
+        const int cost = ((units * k + wave - 1) / wave) * ((blocks + k - 1) / k + kWaveBlocks);
+        if (k == 1 || cost < best) {
+            best = cost;
+            c = k;
+        }
+    }
     a.csize = c;
     a.nb = (blocks + c - 1) / c >= 3 ? 2 : 1;  // long key ranges keep two K/V sub-blocks in flight
     return a;

@@ -77,6 +77,9 @@ def test_wide_head_split_tiles(pkg, V, N, d):
 @pytest.mark.parametrize("B,T,H,Hkv,kv", [
     (1, 5, 28, 4, [1200]), (2, 32, 28, 4, [1024, 3]), (1, 64, 8, 4, [1500]), (1, 43, 6, 2, [1061]),
     (2, 100, 8, 1, [1300, 700]), (3, 96, 4, 4, [2000, 64, 1]), (1, 129, 4, 2, [1111]),
+    # two, three, six and seven key splits
+    (6, 20, 24, 24, [1100, 900, 64, 1, 1003, 500]), (3, 32, 32, 32, [1100, 64, 1]), (1, 64, 8, 8, [1030]),
+    (1, 64, 8, 8, [1200]),
 ])
 def test_group_query_tiles(pkg, B, T, H, Hkv, kv):
     g = torch.Generator().manual_seed(B * T + H)
