@@ -163,6 +163,31 @@ __device__ __forceinline__ void warp_reduce_scatter(float* v, int lane) {
     for (int w = 16 / N; w >= 1; w >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], w);
 }
 
+// The same scattered reduction of (value, index) pairs to the largest value, the smaller index
+// among equals: N-1 + log2(32/N) exchanges of a pair, where a butterfly of every column takes 5 N
+// (160 shuffles for 16 columns: more code than the rest of the LM head's epilogue, run cold).
+template <int N>
+__device__ __forceinline__ void warp_argmax_scatter(float* m, int* idx, int lane) {
+    auto merge = [&](int i, float km, int ki, float om, int oi) {
+        const bool take = om > km || (om == km && oi < ki);
+        m[i] = take ? om : km;
+        idx[i] = take ? oi : ki;
+    };
+#pragma unroll
+    for (int w = 16, h = N / 2; h >= 1; w >>= 1, h >>= 1) {
+        const bool upper = (lane & w) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float om = __shfl_xor_sync(0xffffffffu, upper ? m[i] : m[i + h], w);
+            const int oi = __shfl_xor_sync(0xffffffffu, upper ? idx[i] : idx[i + h], w);
+            merge(i, upper ? m[i + h] : m[i], upper ? idx[i + h] : idx[i], om, oi);
+        }
+    }
+#pragma unroll
+    for (int w = 16 / N; w >= 1; w >>= 1)
+        merge(0, m[0], idx[0], __shfl_xor_sync(0xffffffffu, m[0], w), __shfl_xor_sync(0xffffffffu, idx[0], w));
+}
+
 // What a QKV epilogue thread needs besides the accumulator, from the tile and chunk alone: its
 // row's part (q, K or V) and position in the head, the rotation at its first column and the
 // per-column step (angle addition along the positions, when all 32 columns are consecutive
@@ -400,7 +425,7 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
                 if (gate_lane) st[(GW * g + u) * 64] = hv;
             }
         } else if constexpr (EPI == EPI_LMHEAD) {
-            // this warp's (max, argmax, sum exp) over its 32 rows, for the 8 columns side by side
+            // this warp's (max, argmax, sum exp) over its 32 rows, for the 16 columns side by side
             float m[GW], e[GW];
             int idx[GW];
 #pragma unroll
@@ -408,25 +433,16 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
                 m[u] = lm_ok ? a[u] : -INFINITY;
                 idx[u] = lm_ok ? row : INT_MAX;
             }
+            warp_argmax_scatter<GW>(m, idx, lane);
+            const float mc = m[0];  // of column lane / LS
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-                for (int u = 0; u < GW; ++u) {
-                    const float om = __shfl_xor_sync(0xffffffffu, m[u], off);
-                    const int oi = __shfl_xor_sync(0xffffffffu, idx[u], off);
-                    const bool take = om > m[u] || (om == m[u] && oi < idx[u]);
-                    m[u] = take ? om : m[u];
-                    idx[u] = take ? oi : idx[u];
-                }
+            for (int u = 0; u < GW; ++u) {
+                const float mu = __shfl_sync(0xffffffffu, mc, u * LS);
+                e[u] = (lm_ok && mu != -INFINITY) ? __expf(a[u] - mu) : 0.0f;
             }
-#pragma unroll
-            for (int u = 0; u < GW; ++u) e[u] = (lm_ok && m[u] != -INFINITY) ? __expf(a[u] - m[u]) : 0.0f;
-            if (lane == 0) {
-#pragma unroll
-                for (int u = 0; u < GW; ++u) {
-                    sm.red[(quarter * 32 + GW * g + u) * 3] = m[u];
-                    sm.red[(quarter * 32 + GW * g + u) * 3 + 2] = __int_as_float(idx[u]);
-                }
+            if (lane % LS == 0) {
+                sm.red[(quarter * 32 + GW * g + lane / LS) * 3] = mc;
+                sm.red[(quarter * 32 + GW * g + lane / LS) * 3 + 2] = __int_as_float(idx[0]);
             }
             warp_reduce_scatter<GW>(e, lane);
             if (lane % LS == 0) sm.red[(quarter * 32 + GW * g + lane / LS) * 3 + 1] = e[0];

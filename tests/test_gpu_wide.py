@@ -93,3 +93,27 @@ def test_group_query_tiles(pkg, B, T, H, Hkv, kv):
         got = out.view(B, T, H, 128)[b].transpose(0, 1).double()
         assert (got - ref).norm() <= 1e-2 * ref.norm()  # bf16 probabilities and outputs
         assert (got - ref).abs().max() <= 0.05 * ref.abs().max()
+
+
+@pytest.mark.parametrize("N", [32, 40])
+def test_head_argmax_ties(pkg, N):
+    """Equal largest logits in one warp's rows, in two quarters, in two tiles and beside the mask id:
+    the lowest id wins; conf is exact (the tied logits are 0 or powers of two apart)."""
+    V, d, mask = 384, 64, 5
+    W = torch.zeros(V, d, dtype=torch.bfloat16, device="cuda")
+    X = torch.zeros(N, d, dtype=torch.bfloat16, device="cuda")
+    for k, ids in enumerate([(3, 9), (40, 70), (100, 300), (mask, 7, 8), (383,), (127, 128)]):
+        W[list(ids), k] = 16.0
+    first = [3, 40, 100, 7, 383, 127, 0]  # the last kind: every logit 0
+    ties = [2, 2, 2, 2, 1, 2, V - 1]
+    kind = [n % 7 for n in range(N)]
+    for n, k in enumerate(kind):
+        if k < 6:
+            X[n, k] = 1.0
+    cur = torch.zeros(N, dtype=torch.int32, device="cuda")
+    x0, conf, _, _ = pkg.dllm_op_lmhead(W, X, cur, V, N, d, mask)
+    rest = np.exp(-16.0)
+    for n, k in enumerate(kind):
+        assert int(x0[n]) == first[k]
+        p = 1 / ties[k] if k == 6 else 1 / (ties[k] + (V - 1 - ties[k]) * rest)
+        assert abs(float(conf[n]) - p) <= 1e-5 * p  # a sum of at most 384 exponentials in fp32
