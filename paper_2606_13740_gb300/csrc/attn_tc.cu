@@ -434,7 +434,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // the partial (unnormalised O, max, sum) of rows < nq into shared memory, over the
             // Q/K/V tiles: every copy into them has landed and every MMA reading them is done
             // (the P.V above was the last, and MMAs complete in issue order)
-            float* sO = reinterpret_cast<float*>(smem);  // [128][128]
+            // [128][128], a row's 16-byte pieces at piece ^ (row % 8): a thread stores its row, and
+            // unswizzled the 32 rows of a warp fell into the same banks (2 us of a split unit)
+            float* sO = reinterpret_cast<float*>(smem);
             float* sML = sO + kTcRows * 128;             // [128][2]
 #pragma unroll 1
             for (int c = 0; c < 128; c += 32) {
@@ -446,9 +448,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     for (int i = 0; i < 32; ++i) o[i] = 0.0f;
                 }
                 if (r < nq) {
-                    float4* dst = reinterpret_cast<float4*>(sO + r * 128 + c);
+                    float4* dst = reinterpret_cast<float4*>(sO + r * 128);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) dst[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                    for (int i = 0; i < 8; ++i) dst[(c / 4 + i) ^ (r & 7)] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
                 }
             }
             if (r < nq) *reinterpret_cast<float2*>(sML + r * 2) = make_float2(nsub > 0 ? m : -INFINITY, l);
@@ -467,46 +469,60 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
         for (int c = 0; c < kTcMaxCluster; ++c) pb[c] = c < csize ? dsmem_map_tc(smem_u32(sO), c) : 0u;
         const int nel = nq * 32;
-        for (int ew0 = split * kTcThreads + warp * 32; ew0 < nel; ew0 += csize * kTcThreads) {
-            const int rr = ew0 / 32, i4 = lane;  // one row per warp pass
-            float mk = -INFINITY, lk = 0.0f;
-            if (lane < csize) {
-                const float2 ml = dsmem_ld2_tc(dsmem_map_tc(smem_u32(sML + rr * 2), static_cast<uint32_t>(lane)));
-                mk = ml.x;
-                lk = ml.y;
-            }
-            float4 ov[kTcMaxCluster];
+        // Two rows a pass, their loads all in flight together: a pass costs a round trip through
+        // the cluster.
+        const int step = csize * kTcThreads;
+        for (int ew0 = split * kTcThreads + warp * 32; ew0 < nel; ew0 += 2 * step) {
+            float mk[2], lk[2];
+            float4 ov[2][kTcMaxCluster];
 #pragma unroll
-            for (int c = 0; c < kTcMaxCluster; ++c)
-                if (c < csize) ov[c] = dsmem_ld4_tc(pb[c] + static_cast<uint32_t>((rr * 128 + i4 * 4) * 4));
-            float M = mk;
-            M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 1));
-            M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 2));
-            M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 4));
-            M = __shfl_sync(0xffffffffu, M, 0);
-            const float wk = mk == -INFINITY ? 0.0f : exp2f(mk - M);  // a share without keys: 0
-            float L = wk * lk;
-            L += __shfl_xor_sync(0xffffffffu, L, 1);
-            L += __shfl_xor_sync(0xffffffffu, L, 2);
-            L += __shfl_xor_sync(0xffffffffu, L, 4);
-            L = __shfl_sync(0xffffffffu, L, 0);
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int c = 0; c < kTcMaxCluster; ++c) {
-                if (c < csize) {
-                    const float w = __shfl_sync(0xffffffffu, wk, c);
-                    acc.x += w * ov[c].x;
-                    acc.y += w * ov[c].y;
-                    acc.z += w * ov[c].z;
-                    acc.w += w * ov[c].w;
+            for (int u = 0; u < 2; ++u) {
+                const int rr = min(ew0 + u * step, nel - 32) / 32;  // one row per warp
+                mk[u] = -INFINITY;
+                lk[u] = 0.0f;
+                if (lane < csize) {
+                    const float2 ml = dsmem_ld2_tc(dsmem_map_tc(smem_u32(sML + rr * 2), static_cast<uint32_t>(lane)));
+                    mk[u] = ml.x;
+                    lk[u] = ml.y;
                 }
+#pragma unroll
+                for (int c = 0; c < kTcMaxCluster; ++c)
+                    if (c < csize)
+                        ov[u][c] = dsmem_ld4_tc(pb[c] + static_cast<uint32_t>((rr * 128 + ((lane ^ (rr & 7)) * 4)) * 4));
             }
-            const float inv = L > 0.0f ? 1.0f / L : 0.0f;
-            __nv_bfloat16* op = out + out_off(q0 + rr) + i4 * 4;
-            uint2 w2;
-            w2.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-            w2.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-            *reinterpret_cast<uint2*>(op) = w2;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (ew0 + u * step >= nel) break;
+                const int rr = (ew0 + u * step) / 32;
+                float M = mk[u];
+                M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 1));
+                M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 2));
+                M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 4));
+                M = __shfl_sync(0xffffffffu, M, 0);
+                const float wk = mk[u] == -INFINITY ? 0.0f : exp2f(mk[u] - M);  // a share without keys: 0
+                float L = wk * lk[u];
+                L += __shfl_xor_sync(0xffffffffu, L, 1);
+                L += __shfl_xor_sync(0xffffffffu, L, 2);
+                L += __shfl_xor_sync(0xffffffffu, L, 4);
+                L = __shfl_sync(0xffffffffu, L, 0);
+                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int c = 0; c < kTcMaxCluster; ++c) {
+                    if (c < csize) {
+                        const float w = __shfl_sync(0xffffffffu, wk, c);
+                        acc.x += w * ov[u][c].x;
+                        acc.y += w * ov[u][c].y;
+                        acc.z += w * ov[u][c].z;
+                        acc.w += w * ov[u][c].w;
+                    }
+                }
+                const float inv = L > 0.0f ? 1.0f / L : 0.0f;
+                __nv_bfloat16* op = out + out_off(q0 + rr) + lane * 4;
+                uint2 w2;
+                w2.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+                w2.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+                *reinterpret_cast<uint2*>(op) = w2;
+            }
         }
         if (tr) tr[kTcMergeLoop] = global_ns();
         cluster_sync_tc();  // no CTA leaves while its partial may still be read
