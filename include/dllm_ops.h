@@ -2,8 +2,10 @@
  * dllm_ops.h - single-kernel entry points of the denoising path, for
  * kernel-level parity tests and micro-benchmarks.  Same conventions as
  * dllm.h (0 = OK, negative DLLM_E* codes; messages via dllm_last_error(NULL)).
- * Device pointers are marked "dev"; these calls allocate their own scratch
- * with cudaMalloc and free it before returning, and synchronise the stream.
+ * Device pointers are marked "dev"; these calls allocate their own scratch and
+ * free it before returning (the projections and the LM head from a memory pool
+ * per device that keeps up to 64 MB between calls, ordered by the stream), and
+ * synchronise the stream.
  */
 #ifndef DLLM_OPS_H
 #define DLLM_OPS_H
@@ -19,8 +21,9 @@ extern "C" {
  * paper offloads to the NPU; here tcgen05 tensor cores):
  * D[n][m] = sum_k W[m][k] * X[n][k].  W dev bf16 [M][K] row-major, X dev bf16
  * [N][K] row-major, D dev fp32 [N][M].  K*2 bytes must be a multiple of 16;
- * W and X 16-byte aligned.  grid = CTAs of the stream-K split (0 or more
- * than the SM count: one per SM; the CTAs that finish a split tile wait for
+ * W and X 16-byte aligned.  grid = CTAs of the stream-K split (more
+ * than the SM count: one per SM; 0: the same, or for small operands one per
+ * whole 32-token tile; the CTAs that finish a split tile wait for
  * its other contributors, so all of them must be resident at once).
  * Errors: DLLM_EINVAL, DLLM_ECUDA, DLLM_ETIMEOUT. */
 int dllm_op_gemm(const void* W, const void* X, float* D, int M, int N, int K, int grid, void* stream);
