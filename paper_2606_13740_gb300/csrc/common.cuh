@@ -122,16 +122,9 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* t
         : "memory");
 }
 
-// Bulk copy global -> shared (no tensor map): both addresses 16-byte aligned,
-// bytes a multiple of 16; completion counted in bytes on bar.
-__device__ __forceinline__ void bulk_load(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(smem_dst)),
-                 "l"(reinterpret_cast<uint64_t>(gsrc)), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-// The same with an L2 eviction policy (createpolicy) for the source lines.
+// Bulk copy global -> shared (no tensor map), with an L2 eviction policy (createpolicy) for the
+// source lines: both addresses 16-byte aligned, bytes a multiple of 16; completion counted in
+// bytes on bar.
 __device__ __forceinline__ void bulk_load_hint(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar,
                                                uint64_t policy) {
     asm volatile(

@@ -279,10 +279,11 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
     // col0: the chunk's first token column; c_in: its offset inside the token tile (index into
     // the tile's RMSNorm scales and staged ids).  The thread's 16 accumulator columns come from
     // a_in (a finisher's sum of the parts, in registers), else from TMEM at t_src.  The old
-    // residual (pass 1) comes from TMEM (t_x), else from global memory (a warp's 32 rows of a
-    // token are one 128-byte line; L2 only: other CTAs wrote them in earlier phases); pass 1
-    // leaves the new residual in the accumulator, where pass 2 reads it.  e: the epilogue thread (0 .. kEpiThreads-1), half: which 16 columns of the
-    // chunk.  qkv_pre: the QKV plan, built ahead (null: built here).
+    // residual (pass 1) comes from TMEM (t_x), is in a_in already (x_added), or comes from global
+    // memory (a warp's 32 rows of a token are one 128-byte line; L2 only: other CTAs wrote them in
+    // earlier phases); pass 1 leaves the new residual in the accumulator, where pass 2 reads it.
+    // e: the epilogue thread (0 .. kEpiThreads-1), half: which 16 columns of the chunk.  qkv_pre:
+    // the QKV plan, built ahead (null: built here).  buf: the staging buffer (ALT).
     constexpr int GW = kEpiGroup;  // columns per group
     constexpr int LS = 32 / GW;    // lanes sharing one column's sum after the scatter
     uint8_t* const stg = ALT ? sm.stg + buf * kStgBytes : sm.stg;
