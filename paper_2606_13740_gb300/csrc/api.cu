@@ -699,7 +699,6 @@ static int set_debug_buffers(dllm_ctx* ctx) {
     size_t need = static_cast<size_t>(ctx->L.max_tok) * ctx->cfg.vocab;
     if (ctx->logits_cap >= need) return DLLM_OK;
     if (ctx->logits) cudaFree(ctx->logits);
-    if (ctx->trace) cudaFree(ctx->trace);
     ctx->logits = nullptr;
     if (cudaMalloc(&ctx->logits, need * 4) != cudaSuccess) return fail(ctx, DLLM_ENOMEM, "logits buffer");
     ctx->logits_cap = need;

@@ -324,6 +324,34 @@ def test_rewind_repeats_identical_step(model):
     ctx.close()
 
 
+def test_trace_and_logits_together(model):
+    """The timeline buffer outlives the logits buffer made after it, in one call and in two: the
+    kernels' stamps are there, in this step's order, and the logits are those without a timeline."""
+    from paper_2606_13740_gb300 import Sched
+    prompt = I.uniform_prompt(32, TINY.vocab, TINY.mask_id, seed=5)
+
+    def run(*flags):
+        ctx = _gpu_ctx()
+        for f in flags:
+            ctx.dllm_set_debug(f)
+        ctx.dllm_prefill(Sched(), prompt, 32)
+        ctx.dllm_begin_block()
+        ctx.dllm_denoise_step()
+        lg, tr = ctx.dllm_get_step_debug(logits=True)["logits"], ctx.dllm_get_trace() if flags[-1] & 16 else None
+        ctx.close()
+        return lg, tr
+
+    plain, _ = run(1)
+    for flags in ((17,), (16, 17)):
+        lg, tr = run(*flags)
+        assert np.array_equal(lg, plain)
+        # the first projection, then a layer's attention and its chain's four phases
+        assert len(tr) == 1 + 5 * TINY.n_layers
+        chain = [0] + [2 + 5 * l + i for l in range(TINY.n_layers) for i in range(4)]
+        start, done = (tr[chain, 0, s].astype(np.int64) for s in (0, 4))  # of CTA 0
+        assert (start > 0).all() and (done >= start).all() and (np.diff(done) >= 0).all()
+
+
 def test_errors_poison_context(model):
     """Argument and capacity errors leave the context usable; a device-side failure (here a
     bounded wait that runs out) poisons it: the call reports DLLM_ETIMEOUT, every later call
