@@ -38,8 +38,8 @@ int sm_count() {
 // one per device, so that a call does not pay for cudaMalloc and cudaFree (about 250 us for the
 // 40 MB of split partials of a 1024-token projection, beside 150 us on the GPU).  Allocation and
 // release are ordered by the call's stream, which makes the pool safe for calls on several
-// streams and from several threads; between calls it keeps at most kPoolKeepBytes and gives the
-// rest back to the device.
+// streams and from several threads.  A call releases its scratch before it waits for its stream:
+// a wait is where a pool gives back to the device what it holds past kPoolKeepBytes.
 constexpr uint64_t kPoolKeepBytes = uint64_t(64) << 20;
 constexpr int kMaxDevices = 64;
 
@@ -71,8 +71,11 @@ struct OpScratch {
     uint8_t* p = nullptr;
     cudaStream_t st = nullptr;
     size_t used = 0;
-    ~OpScratch() {
-        if (p) cudaFreeAsync(p, st);
+    ~OpScratch() { release(); }
+    cudaError_t release() {
+        void* q = p;
+        p = nullptr;
+        return q ? cudaFreeAsync(q, st) : cudaSuccess;
     }
     static size_t rounded(size_t bytes) { return (bytes + 255) / 256 * 256; }
     bool alloc(size_t bytes, size_t zero_bytes, cudaStream_t stream) {
@@ -106,9 +109,11 @@ struct DevBuf {
     bool alloc(size_t bytes) { return cudaMalloc(&p, bytes ? bytes : 16) == cudaSuccess; }
 };
 
-int finish(cudaStream_t st, int* status_dev) {
+// Waits for a call's kernels and reports; buf: its scratch, of which status_dev is a part.
+int finish(cudaStream_t st, int* status_dev = nullptr, OpScratch* buf = nullptr) {
     int s = 0;
     cudaError_t e = status_dev ? cudaMemcpyAsync(&s, status_dev, 4, cudaMemcpyDeviceToHost, st) : cudaSuccess;
+    if (e == cudaSuccess && buf) e = buf->release();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return op_fail(DLLM_ECUDA, "%s", cudaGetErrorString(e));
     if (s & kStatusTimeout) return op_fail(DLLM_ETIMEOUT, "bounded device wait ran out");
@@ -154,10 +159,9 @@ static int gemm_impl(const void* W, const void* X, float* D, int M, int N, int K
     if (flags & 4) {
         // the bounded-wait test: one launch whose operand producer waits for a word nobody
         // writes (the zeroed third int of the status allocation; the launch's tag is 1)
-        cudaError_t e = gemm_launch(EPI_F32, p, tw, tx, ep, scr, status, st,
-                                    status + 2);
+        cudaError_t e = gemm_launch(EPI_F32, p, tw, tx, ep, scr, status, st, status + 2);
         if (e != cudaSuccess) return op_fail(DLLM_ECUDA, "gemm launch: %s", cudaGetErrorString(e));
-        return finish(st, status);
+        return finish(st, status, &buf);
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ms && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))
@@ -176,7 +180,7 @@ static int gemm_impl(const void* W, const void* X, float* D, int M, int N, int K
     if (ms && e == cudaSuccess) e = cudaEventRecord(e1, st);
     int rc = DLLM_OK;
     if (e != cudaSuccess) rc = op_fail(DLLM_ECUDA, "gemm launch: %s", cudaGetErrorString(e));
-    if (rc == DLLM_OK) rc = finish(st, status);
+    if (rc == DLLM_OK) rc = finish(st, status, &buf);
     if (rc == DLLM_OK && ms) {
         float t = 0.0f;
         cudaEventElapsedTime(&t, e0, e1);
@@ -223,7 +227,7 @@ int dllm_op_attention(const void* q, const void* kc, const void* vc, const int32
                                      static_cast<const __nv_bfloat16*>(vc), kv_len, static_cast<__nv_bfloat16*>(out),
                                      B, T, H, Hkv, hd, cap, a, st, false);
     if (e != cudaSuccess) return op_fail(DLLM_ECUDA, "attention launch: %s", cudaGetErrorString(e));
-    return finish(st, nullptr);
+    return finish(st);
 }
 
 int dllm_op_lmhead(const void* W, const void* X, const int32_t* cur, int32_t* x0, float* conf, float* tokconf,
@@ -262,10 +266,9 @@ int dllm_op_lmhead(const void* W, const void* X, const int32_t* cur, int32_t* x0
     ep.mask_id = mask_id;
     cudaError_t e = gemm_launch(EPI_LMHEAD, p, tw, tx, ep, scr, status, st);
     if (e == cudaSuccess)
-        e = launch_lmhead_reduce(lmp, zc, cur, p.m_tiles, N, mask_id, x0,
-                                 conf, tokconf, st, false);
+        e = launch_lmhead_reduce(lmp, zc, cur, p.m_tiles, N, mask_id, x0, conf, tokconf, st, false);
     if (e != cudaSuccess) return op_fail(DLLM_ECUDA, "lmhead launch: %s", cudaGetErrorString(e));
-    return finish(st, status);
+    return finish(st, status, &buf);
 }
 
 int dllm_op_commit(int32_t* tok, uint8_t* status, int n_pos, int w0, int T, int c0, int c1, int step,

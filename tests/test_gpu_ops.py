@@ -143,6 +143,27 @@ def test_lmhead_decision_matches_oracle(dev, V, N, d, mask):
         assert abs(tc[n] - rtc) <= 1e-3 * max(rtc, 1e-30) + 1e-12
 
 
+def test_call_scratch_kept_is_bounded(dev):
+    """A call whose scratch passes 64 MB (here 97 MB of LM-head statistics, and its partials) has
+    given back what is beyond that when it returns, with no synchronisation by the caller."""
+    from paper_2606_13740_gb300 import dllm_op_lmhead
+    V, N, d = 126464, 8192, 256
+    W = torch.zeros(V, d, dtype=torch.bfloat16, device=dev)
+    X = torch.zeros(N, d, dtype=torch.bfloat16, device=dev)
+    cur = torch.zeros(N, dtype=torch.int32, device=dev)
+    dllm_op_lmhead(W, X, cur, 1024, 64, d, 0)  # code loaded
+    outputs = [torch.empty(N, device=dev) for _ in range(3)]
+    del outputs  # their memory stays at hand
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    x0, conf, _, _ = dllm_op_lmhead(W, X, cur, V, N, d, 0)
+    kept = free - torch.cuda.mem_get_info()[0]
+    assert kept <= 64 << 20, kept
+    # equal logits, the mask id 0 left out: the lowest other id, one of V - 1 alike (an fp32 sum
+    # of V - 1 ones is exact below 2^24)
+    assert bool((x0 == 1).all()) and bool(((conf * (V - 1) - 1).abs() <= 1e-6).all())
+
+
 # ------------------------------------------------------------------ commit
 def _random_case(rng, use_cache, spec_blocks):
     bl = 32
