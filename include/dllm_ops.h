@@ -3,9 +3,9 @@
  * kernel-level parity tests and micro-benchmarks.  Same conventions as
  * dllm.h (0 = OK, negative DLLM_E* codes; messages via dllm_last_error(NULL)).
  * Device pointers are marked "dev"; these calls allocate their own scratch and
- * free it before returning, and synchronise the stream.  The projections and
- * the LM head take it, ordered by the stream, from a memory pool per device
- * that keeps up to 64 MB when a call returns.
+ * free it before returning, and synchronise the stream.  Of the scratch of the
+ * projections and the LM head up to 64 MB stay allocated for the next call, per
+ * context and as long as the context.
  */
 #ifndef DLLM_OPS_H
 #define DLLM_OPS_H

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -34,67 +35,136 @@ int sm_count() {
     return n;
 }
 
-// The scratch of the projection and LM-head calls comes from a memory pool of this library's,
-// one per device, so that a call does not pay for cudaMalloc and cudaFree (about 250 us for the
-// 40 MB of split partials of a 1024-token projection, beside 150 us on the GPU).  Allocation and
-// release are ordered by the call's stream, which makes the pool safe for calls on several
-// streams and from several threads.  A call releases its scratch before it waits for its stream:
-// a wait is where a pool gives back to the device what it holds past kPoolKeepBytes.
-constexpr uint64_t kPoolKeepBytes = uint64_t(64) << 20;
-constexpr int kMaxDevices = 64;
+// The scratch of the projection and LM-head calls is kept from one call for the next, so that a
+// call does not pay for cudaMalloc and cudaFree (about 250 us for the 40 MB of split partials of a
+// 1024-token projection, beside 150 us on the GPU).  A call takes a kept buffer for itself alone
+// and puts it back once it has waited for its kernels, so calls on several streams and from
+// several threads never share one.  At most kKeepBytes stay kept for a context.  The buffers are
+// plain cudaMalloc memory of their context and end with it (cudaDeviceReset): a buffer is found
+// again only under its context's id, which the process never gives out twice.
+constexpr size_t kKeepBytes = size_t(64) << 20;
 
-cudaMemPool_t scratch_pool() {
-    static std::mutex mu;
-    static cudaMemPool_t pools[kMaxDevices] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!pools[dev]) {
-        cudaMemPoolProps props{};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t pool = nullptr;
-        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) return nullptr;
-        uint64_t keep = kPoolKeepBytes;
-        if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaMemPoolDestroy(pool);
-            return nullptr;
-        }
-        pools[dev] = pool;
-    }
-    return pools[dev];
+struct KeptBuf {
+    unsigned long long ctx;
+    void* p;
+    size_t bytes;
+    KeptBuf* next;
+};
+std::mutex kept_mu;
+KeptBuf* kept = nullptr;  // under kept_mu
+
+// The id of the current context (which the caller has made by an earlier call to the runtime).
+bool current_context(unsigned long long* id) {
+    typedef CUresult (*GetIdFn)(CUcontext, unsigned long long*);
+    static const GetIdFn get_id = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &q);
+        return reinterpret_cast<GetIdFn>(e == cudaSuccess && q == cudaDriverEntryPointSuccess ? fn : nullptr);
+    }();
+    return get_id && get_id(nullptr, id) == CUDA_SUCCESS;
 }
 
-// One call's scratch, carved from one allocation: zeroed pieces first, then the others.
+// Frees a list of buffers of the current context.
+void free_bufs(KeptBuf* b) {
+    while (b) {
+        KeptBuf* next = b->next;
+        cudaFree(b->p);
+        delete b;
+        b = next;
+    }
+}
+
+// Takes the smallest kept buffers of a context off the list until the others hold `bytes` at most.
+KeptBuf* drop_past(unsigned long long ctx, size_t bytes) {  // under kept_mu
+    KeptBuf* out = nullptr;
+    for (;;) {
+        size_t sum = 0;
+        KeptBuf** least = nullptr;
+        for (KeptBuf** e = &kept; *e; e = &(*e)->next) {
+            if ((*e)->ctx != ctx) continue;
+            sum += (*e)->bytes;
+            if (!least || (*e)->bytes < (*least)->bytes) least = e;
+        }
+        if (sum <= bytes) return out;
+        KeptBuf* b = *least;
+        *least = b->next;
+        b->next = out;
+        out = b;
+    }
+}
+
+// A buffer of at least `bytes`: the smallest kept one that does, else a new one (where memory is
+// short, in the place of the kept ones); null: no memory.
+KeptBuf* take_buf(size_t bytes) {
+    unsigned long long ctx = 0;
+    if (!current_context(&ctx)) return nullptr;
+    {
+        std::lock_guard<std::mutex> lock(kept_mu);
+        KeptBuf** best = nullptr;
+        for (KeptBuf** e = &kept; *e; e = &(*e)->next)
+            if ((*e)->ctx == ctx && (*e)->bytes >= bytes && (!best || (*e)->bytes < (*best)->bytes)) best = e;
+        if (best) {
+            KeptBuf* b = *best;
+            *best = b->next;
+            b->next = nullptr;
+            return b;
+        }
+    }
+    KeptBuf* b = new (std::nothrow) KeptBuf{ctx, nullptr, bytes, nullptr};
+    if (!b) return nullptr;
+    if (cudaMalloc(&b->p, bytes) == cudaSuccess) return b;
+    cudaGetLastError();
+    KeptBuf* out;
+    {
+        std::lock_guard<std::mutex> lock(kept_mu);
+        out = drop_past(ctx, 0);
+    }
+    const bool more = out != nullptr;
+    free_bufs(out);
+    if (more && cudaMalloc(&b->p, bytes) == cudaSuccess) return b;
+    cudaGetLastError();
+    delete b;
+    return nullptr;
+}
+
+// Keeps a buffer that no work uses any more, smaller ones dropped where that is too much.
+void keep_buf(KeptBuf* b) {
+    KeptBuf* out = b;
+    if (b->bytes <= kKeepBytes) {
+        std::lock_guard<std::mutex> lock(kept_mu);
+        out = drop_past(b->ctx, kKeepBytes - b->bytes);
+        b->next = kept;
+        kept = b;
+    }
+    free_bufs(out);
+}
+
+// One call's scratch, carved from one buffer: zeroed pieces first, then the others.
 struct OpScratch {
-    uint8_t* p = nullptr;
-    cudaStream_t st = nullptr;
+    KeptBuf* buf = nullptr;
     size_t used = 0;
-    ~OpScratch() { release(); }
-    cudaError_t release() {
-        void* q = p;
-        p = nullptr;
-        return q ? cudaFreeAsync(q, st) : cudaSuccess;
+    bool idle = false;  // the call's work on it is done
+    ~OpScratch() {
+        if (!buf) return;
+        if (idle) keep_buf(buf);
+        else free_bufs(buf);
     }
     static size_t rounded(size_t bytes) { return (bytes + 255) / 256 * 256; }
-    bool alloc(size_t bytes, size_t zero_bytes, cudaStream_t stream) {
-        st = stream;
+    bool alloc(size_t bytes, size_t zero_bytes, cudaStream_t st) {
+        // The calls synchronise, so they are refused, before anything is launched or captured, on a
+        // capturing stream and where another stream's capture forbids this thread such calls (the
+        // query is one of those).
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        // the calls synchronise, so they are refused on a capturing stream, before anything is captured
         if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-        cudaMemPool_t pool = scratch_pool();
-        void* q = nullptr;
-        if (!pool || cudaMallocFromPoolAsync(&q, bytes, pool, st) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        p = static_cast<uint8_t*>(q);
-        return cudaMemsetAsync(p, 0, zero_bytes, st) == cudaSuccess;
+        const cudaError_t query = cudaStreamQuery(st);
+        if (query != cudaSuccess && query != cudaErrorNotReady) return false;
+        buf = take_buf(bytes);
+        return buf && cudaMemsetAsync(buf->p, 0, zero_bytes, st) == cudaSuccess;
     }
     template <typename T>
     T* take(size_t bytes) {
-        T* q = reinterpret_cast<T*>(p + used);
+        T* q = reinterpret_cast<T*>(static_cast<uint8_t*>(buf->p) + used);
         used += rounded(bytes);
         return q;
     }
@@ -113,8 +183,8 @@ struct DevBuf {
 int finish(cudaStream_t st, int* status_dev = nullptr, OpScratch* buf = nullptr) {
     int s = 0;
     cudaError_t e = status_dev ? cudaMemcpyAsync(&s, status_dev, 4, cudaMemcpyDeviceToHost, st) : cudaSuccess;
-    if (e == cudaSuccess && buf) e = buf->release();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (buf) buf->idle = e == cudaSuccess;
     if (e != cudaSuccess) return op_fail(DLLM_ECUDA, "%s", cudaGetErrorString(e));
     if (s & kStatusTimeout) return op_fail(DLLM_ETIMEOUT, "bounded device wait ran out");
     if (s) return op_fail(DLLM_ECUDA, "device status %d", s);

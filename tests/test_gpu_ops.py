@@ -164,6 +164,43 @@ def test_call_scratch_kept_is_bounded(dev):
     assert bool((x0 == 1).all()) and bool(((conf * (V - 1) - 1).abs() <= 1e-6).all())
 
 
+_RESET = """
+import ctypes as C, sys
+import numpy as np, torch
+from paper_2606_13740_gb300 import dllm
+rt = C.CDLL("libcudart.so." + torch.version.cuda.split(".")[0])  # the one torch has loaded
+M, N, K = 256, 40, 512
+w, x = (np.random.default_rng(i).integers(0, 2, (r, K)).astype(np.uint16) for i, r in enumerate((M, N)))
+ref = x.astype(np.float32) @ w.astype(np.float32).T
+free, total = C.c_size_t(), C.c_size_t()
+left = []
+for _ in range(4):
+    p = [C.c_void_p() for _ in range(3)]
+    d = np.zeros((N, M), np.float32)
+    for q, a in zip(p, (w * 0x3F80, x * 0x3F80, d)):  # bf16 ones
+        assert rt.cudaMalloc(C.byref(q), C.c_size_t(a.nbytes)) == 0
+        assert rt.cudaMemcpy(q, a.ctypes.data_as(C.c_void_p), C.c_size_t(a.nbytes), 1) == 0
+    dllm._check(dllm.lib().dllm_op_gemm(*p, M, N, K, 0, None))
+    assert rt.cudaMemcpy(d.ctypes.data_as(C.c_void_p), p[2], C.c_size_t(d.nbytes), 2) == 0
+    assert np.array_equal(d, ref)
+    assert rt.cudaMemGetInfo(C.byref(free), C.byref(total)) == 0
+    left.append(free.value)
+    assert rt.cudaDeviceReset() == 0
+assert len(set(left)) == 1, left  # nothing of an ended context stays behind
+"""
+
+
+def test_calls_survive_a_device_reset(dev):
+    """A projection (its scratch from a pool) after each of several cudaDeviceReset calls, in a
+    process of its own."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _RESET], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+
+
 # ------------------------------------------------------------------ commit
 def _random_case(rng, use_cache, spec_blocks):
     bl = 32
