@@ -5,7 +5,7 @@
  * Device pointers are marked "dev"; these calls allocate their own scratch and
  * free it before returning, and synchronise the stream.  Of the scratch of the
  * projections and the LM head up to 64 MB stay allocated for the next call, per
- * context and as long as the context.
+ * context, until dllm_op_release_scratch or the end of the context.
  */
 #ifndef DLLM_OPS_H
 #define DLLM_OPS_H
@@ -94,6 +94,10 @@ int dllm_op_attention(const void* q, const void* kc, const void* vc, const int32
  * logits dev fp32 [N][V] or NULL. */
 int dllm_op_lmhead(const void* W, const void* X, const int32_t* cur, int32_t* x0, float* conf, float* tokconf,
                    float* logits, int V, int N, int d, int mask_id, void* stream);
+
+/* Frees the scratch that calls have kept for the next one in the current context
+ * (calls in progress go on; the next one allocates anew). */
+void dllm_op_release_scratch(void);
 
 /* One commit / re-mask / draft pass on HOST arrays of one sequence
  * (Sec. 2.1 commit, Sec. 3.2 drafts, Sec. 3.3 revision and staged token

@@ -11,5 +11,5 @@ from .build import build  # noqa: F401
 from .dllm import (  # noqa: F401
     COMMIT_SCHEDULE, COMMIT_THRESHOLD, COMMITTED, DRAFT, FIXED, MASKED, STABLE, Config, Context, DllmError, Sched,
     dllm_arena_bytes, dllm_op_attention,
-    dllm_op_commit, dllm_op_gemm, dllm_op_lmhead, lib,
+    dllm_op_commit, dllm_op_gemm, dllm_op_lmhead, dllm_op_release_scratch, lib,
 )

@@ -602,7 +602,9 @@ int dllm_init(const dllm_config* cfg, void* dev_arena, size_t arena_bytes, void*
             return bail(DLLM_EINVAL, "arena too small or not 256-byte aligned");
         ctx->arena = static_cast<uint8_t*>(dev_arena);
     } else {
-        if (cudaMalloc(&ctx->arena, L.total) != cudaSuccess) return bail(DLLM_ENOMEM, "device allocation failed");
+        if (cudaMalloc(&ctx->arena, L.total) != cudaSuccess &&
+            !(free_kept_scratch() && cudaMalloc(&ctx->arena, L.total) == cudaSuccess))
+            return bail(DLLM_ENOMEM, "device allocation failed");
         ctx->own_arena = true;
     }
     if (gemm_init_attrs() != cudaSuccess || attn_init_attrs() != cudaSuccess || chain_init_attrs() != cudaSuccess)

@@ -15,6 +15,9 @@ constexpr int kMaxBlock = 4096;
 constexpr int kStatusTimeout = 1;  // device status word bits
 constexpr int kStatusBadIndex = 2;  // longest current block the commit pass handles
 
+// Frees the scratch that the single-kernel calls keep in the current context; false: there is none.
+bool free_kept_scratch();
+
 // ---------------------------------------------------------------- weight storage
 // The context's projection weights are stored tile-major: the 128-row x 64-column tile
 // (m-tile r/128, k-block c/64) of a [rows][K] matrix is 16 KB at ((r/128)*kb + c/64)*8192

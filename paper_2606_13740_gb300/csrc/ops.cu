@@ -94,6 +94,23 @@ KeptBuf* drop_past(unsigned long long ctx, size_t bytes) {  // under kept_mu
     }
 }
 
+}  // namespace
+
+bool dllm::free_kept_scratch() {
+    unsigned long long ctx = 0;
+    if (!current_context(&ctx)) return false;
+    KeptBuf* out;
+    {
+        std::lock_guard<std::mutex> lock(kept_mu);
+        out = drop_past(ctx, 0);
+    }
+    const bool any = out != nullptr;
+    free_bufs(out);
+    return any;
+}
+
+namespace {
+
 // A buffer of at least `bytes`: the smallest kept one that does, else a new one (where memory is
 // short, in the place of the kept ones); null: no memory.
 KeptBuf* take_buf(size_t bytes) {
@@ -115,14 +132,7 @@ KeptBuf* take_buf(size_t bytes) {
     if (!b) return nullptr;
     if (cudaMalloc(&b->p, bytes) == cudaSuccess) return b;
     cudaGetLastError();
-    KeptBuf* out;
-    {
-        std::lock_guard<std::mutex> lock(kept_mu);
-        out = drop_past(ctx, 0);
-    }
-    const bool more = out != nullptr;
-    free_bufs(out);
-    if (more && cudaMalloc(&b->p, bytes) == cudaSuccess) return b;
+    if (free_kept_scratch() && cudaMalloc(&b->p, bytes) == cudaSuccess) return b;
     cudaGetLastError();
     delete b;
     return nullptr;
@@ -340,6 +350,8 @@ int dllm_op_lmhead(const void* W, const void* X, const int32_t* cur, int32_t* x0
     if (e != cudaSuccess) return op_fail(DLLM_ECUDA, "lmhead launch: %s", cudaGetErrorString(e));
     return finish(st, status, &buf);
 }
+
+void dllm_op_release_scratch(void) { free_kept_scratch(); }
 
 int dllm_op_commit(int32_t* tok, uint8_t* status, int n_pos, int w0, int T, int c0, int c1, int step,
                    const int32_t* x0, const float* conf, const float* tokconf, int steps_per_block,

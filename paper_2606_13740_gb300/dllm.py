@@ -88,6 +88,7 @@ SIGNATURES = {
     "dllm_op_gemm_timed": (_I, [_P, _P, _P, _I, _I, _I, _I, _I, _I, _P, _P]),
     "dllm_op_attention": (_I, [_P, _P, _P, _P, _P, _I, _I, _I, _I, _I, _I, _I, _P]),
     "dllm_op_lmhead": (_I, [_P, _P, _P, _P, _P, _P, _P, _I, _I, _I, _I, _P]),
+    "dllm_op_release_scratch": (None, []),
     "dllm_op_commit": (_I, [_P, _P, _I, _I, _I, _I, _I, _I, _P, _P, _P, _I, _F, _F, _I, _I, _I, _I, _I, _I, _F, _P]),
 }
 
@@ -420,6 +421,11 @@ def dllm_op_lmhead(W, X, cur, V, N, d, mask_id, want_logits=False, stream=None):
                                 _p(conf.data_ptr()), _p(tc.data_ptr()), _p(None if lg is None else lg.data_ptr()),
                                 V, N, d, mask_id, _p(_stream_ptr(stream))))
     return x0, conf, tc, lg
+
+
+def dllm_op_release_scratch():
+    """Frees the scratch that the calls above have kept for the next one."""
+    lib().dllm_op_release_scratch()
 
 
 def dllm_op_commit(sched: Sched, mask_id, tok, st, w0, T, c0, c1, step, x0, conf, tokconf, block_len=32):
