@@ -26,7 +26,9 @@ using namespace dllm;
 
 namespace {
 
-constexpr int kMaxSMs = 256;  // upper bound for scratch sizing
+// The SMs that a context uses at most, for scratch sizing: the whole die pair of an sm_103a GPU has
+// 160 (a GB300 has 152 of them enabled).
+constexpr int kMaxSMs = 160;
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 int rup(int x, int m) { return (x + m - 1) / m * m; }

@@ -53,6 +53,15 @@ def test_arena_bytes_and_config_checks():
         dllm_arena_bytes(Config(max_batch=64, max_window=128))
 
 
+def test_arena_scratch_is_bounded():
+    """Split partials are a context's largest scratch: four phases of two 128 x 256 fp32 partials for
+    each of 160 CTAs, 160 MiB, where the tokens fill a 256-token tile; less below, no more above."""
+    from paper_2606_13740_gb300 import Config, dllm_arena_bytes
+    mib = {w: dllm_arena_bytes(Config(max_ctx=4096, max_window=w)) / 2**20 for w in (32, 64, 256, 1024)}
+    rest = 32  # weights, cache, activations
+    assert mib[32] <= 10 + rest and mib[64] <= 40 + rest and mib[256] <= 160 + rest and mib[1024] <= 160 + rest
+
+
 def test_init_without_gpu_reports_cuda_error():
     torch = pytest.importorskip("torch")
     if torch.cuda.is_available():
