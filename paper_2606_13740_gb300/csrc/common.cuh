@@ -39,12 +39,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ------------------------------------------------------------------ flags between CTAs
-// Release increment (no return value): orders every write that precedes it, including
-// the writes of other threads of the CTA made before a barrier with this thread.
-__device__ __forceinline__ void red_release_add(int* p, int v) {
-    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-// Counts v in and returns the count before: acquires what the earlier counts released.
+// Counts v in and returns the count before: releases what precedes it (of the other threads too, up
+// to a barrier with this one), acquires what the earlier counts released.
 __device__ __forceinline__ int atom_acq_rel_add(int* p, int v) {
     int old;
     asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
@@ -286,19 +282,6 @@ __device__ __forceinline__ void tmem_ld_32x64(uint32_t taddr, float* v) {
     for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 32 TMEM lanes x 4 consecutive columns -> 4 registers per thread.
-__device__ __forceinline__ void tmem_ld_32x4(uint32_t taddr, float* v) {
-    uint32_t r0, r1, r2, r3;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    v[0] = __uint_as_float(r0);
-    v[1] = __uint_as_float(r1);
-    v[2] = __uint_as_float(r2);
-    v[3] = __uint_as_float(r3);
-}
-
 __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, float* v) {
     uint32_t r[16];
     asm volatile(
@@ -395,8 +378,6 @@ __device__ __forceinline__ bool named_bar_any(int id, int count, bool pred) {
         : "memory");
     return r != 0;
 }
-
-__device__ __forceinline__ bool elect_lane0() { return (threadIdx.x & 31) == 0; }
 
 // One lane of the converged warp, chosen by elect.sync: the issuing thread of a loop the whole
 // warp runs, so that the addresses and descriptors it passes stay warp-uniform values.

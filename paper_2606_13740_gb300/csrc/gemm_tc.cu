@@ -260,33 +260,32 @@ __device__ __forceinline__ QkvPlan qkv_plan(const EpiArgs& ep, const GemmPlan& p
 }
 
 // Epilogue of a 32-token chunk, compact: each epilogue thread takes its TMEM lane (tile row)
-// and one half of the chunk, 16 columns read from TMEM (t_src; for the residual, the old x of
-// a narrow tile was staged at t_x before the accumulator was ready), so its code stays small
-// and no global load waits on a store.  The 16 columns run side by side with no branch between
+// and one half of the chunk, 16 columns, so its code stays small and no global load waits on a
+// store.  The 16 columns run side by side with no branch between
 // them (stores are predicated), so their dependent chains (shuffles, special functions)
 // overlap; the chunk's outputs are staged in shared memory and stored in 16-byte pieces.
-// Residual epilogue in two passes (PASS 1: the bf16 copy, the next projection's operand, and
-// the RMSNorm partial sums; PASS 2: the fp32 residual and the sums' store), so the tile can be
-// published to the next phase's operand producer between them; PASS 0: both at once.
-// ALT: the caller alternates between two staging buffers, so that the barrier between a chunk's
+// The residual epilogue runs in two passes (PASS 1: the bf16 copy, the next projection's operand,
+// and the RMSNorm partial sums; PASS 2: the fp32 residual and the sums' store), so the tile can be
+// published to the next phase's operand producer between them; the others in one (PASS 0).
+// WIDE: the caller alternates between two staging buffers, so that the barrier between a chunk's
 // staging and its stores also covers the buffer's next use.
-template <int EPI, int PASS = 0, bool ALT = false>
+template <int EPI, int PASS = 0, bool WIDE = false>
 __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& p, int mt, int col0, int c_in,
                                              int rt, uint32_t t_src, uint32_t t_x, const EpiSmem& sm,
                                              int e, int half, int quarter, int lane, int* status,
                                              const float* a_in = nullptr, const QkvPlan* qkv_pre = nullptr,
-                                             bool x_added = false, int buf = 0) {
+                                             int buf = 0) {
+    static_assert((EPI == EPI_RESID) == (PASS != 0), "the residual epilogue runs in passes 1 and 2");
     // col0: the chunk's first token column; c_in: its offset inside the token tile (index into
     // the tile's RMSNorm scales and staged ids).  The thread's 16 accumulator columns come from
-    // a_in (a finisher's sum of the parts, in registers), else from TMEM at t_src.  The old
-    // residual (pass 1) comes from TMEM (t_x), is in a_in already (x_added), or comes from global
-    // memory (a warp's 32 rows of a token are one 128-byte line; L2 only: other CTAs wrote them in
-    // earlier phases); pass 1 leaves the new residual in the accumulator, where pass 2 reads it.
+    // a_in (a finisher's sum of the parts, in registers), else from TMEM at t_src.  Pass 1 finds
+    // the old residual in a_in already (WIDE) or in TMEM, staged at t_x, and leaves the new one in
+    // the accumulator, where pass 2 reads it.
     // e: the epilogue thread (0 .. kEpiThreads-1), half: which 16 columns of the chunk.  qkv_pre:
-    // the QKV plan, built ahead (null: built here).  buf: the staging buffer (ALT).
+    // the QKV plan, built ahead (null: built here).  buf: the staging buffer (WIDE).
     constexpr int GW = kEpiGroup;  // columns per group
     constexpr int LS = 32 / GW;    // lanes sharing one column's sum after the scatter
-    uint8_t* const stg = ALT ? sm.stg + buf * kStgBytes : sm.stg;
+    uint8_t* const stg = WIDE ? sm.stg + buf * kStgBytes : sm.stg;
     const int row = mt * kBM + rt;
     const bool scale = (EPI == EPI_QKV || EPI == EPI_SWIGLU || EPI == EPI_LMHEAD) && ep.sq_in != nullptr;
     QkvPlan qp;
@@ -331,21 +330,11 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
                 if (row < p.M && cg + u < p.N) ep.out[static_cast<size_t>(cg + u) * ep.ld_out + row] = a[u];
         } else if constexpr (EPI == EPI_RESID) {
             float xo[GW], ss[GW];
-            if constexpr (PASS == 2) {
+            if constexpr (PASS == 2 || WIDE) {
 #pragma unroll
                 for (int u = 0; u < GW; ++u) xo[u] = a[u];
             } else {
-                if (t_x) {
-                    tmem_ld_32xn<GW>(t_x + static_cast<uint32_t>(GW * g), xo);
-                } else if (x_added) {
-#pragma unroll
-                    for (int u = 0; u < GW; ++u) xo[u] = 0.0f;
-                } else {
-#pragma unroll
-                    for (int u = 0; u < GW; ++u)
-                        xo[u] = (row < p.M && cg + u < p.N) ? __ldcg(ep.out + static_cast<size_t>(cg + u) * ep.ld_out + row)
-                                                            : 0.0f;
-                }
+                tmem_ld_32xn<GW>(t_x + static_cast<uint32_t>(GW * g), xo);
 #pragma unroll
                 for (int u = 0; u < GW; ++u) xo[u] += a[u];
             }
@@ -354,24 +343,18 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
             for (int u = 0; u < GW; ++u) {
                 const bool ok = row < p.M && cg + u < p.N;
                 ss[u] = ok ? xo[u] * xo[u] : 0.0f;
-                if constexpr (PASS == 0) {
-                    if (ok) {
-                        const size_t o = static_cast<size_t>(cg + u) * ep.ld_out + row;
-                        ep.out[o] = xo[u];
-                        ep.xb[o] = __float2bfloat16_rn(xo[u]);
-                    }
-                } else if constexpr (PASS == 1) {  // token-major staging, stored below in 16-byte pieces
+                if constexpr (PASS == 1) {  // token-major staging, stored below in 16-byte pieces
                     reinterpret_cast<__nv_bfloat16*>(stg)[(GW * g + u) * kBM + rt] = __float2bfloat16_rn(xo[u]);
                 } else {  // fp32: a warp's 32 rows of one token are one 128-byte line
                     if (ok) ep.out[static_cast<size_t>(cg + u) * ep.ld_out + row] = xo[u];
                 }
             }
-            if constexpr (PASS != 2) {
+            if constexpr (PASS == 1) {
                 warp_reduce_scatter<GW>(ss, lane);
                 if (lane % LS == 0) sm.red[(c_in / 32) * 128 + quarter * 32 + GW * g + lane / LS] = ss[0];
             }
         } else if constexpr (EPI == EPI_QKV) {
-            // positions and rotations of the group's 8 columns first (the rare tile that spans
+            // positions and rotations of the thread's 16 columns first (the rare tile that spans
             // sequences takes the out-of-line sincos per column), then the branch-free column pass
             int bs[GW], ts[GW];
             float cs[GW], ss[GW];
@@ -466,7 +449,7 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
             for (int i = 0; i < 2; ++i) qp.dst[i] = src[i];
         }
         if (qp.bad) atomicOr(status, kStatusBadIndex);
-        if (!ALT) named_bar(1, kEpiThreads);  // the staging memory is free again
+        if (!WIDE) named_bar(1, kEpiThreads);  // the staging memory is free again
     } else if constexpr (EPI == EPI_SWIGLU) {
         // thread t stores token t/8, features 8 (t%8) .. +7 of the tile's 64
         named_bar(1, kEpiThreads);
@@ -478,7 +461,7 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
             const int fg = mt * 64 + f0;  // F is a multiple of 8: each 8-feature piece is all in or all out
             if (fg < ep.F) *reinterpret_cast<uint4*>(ep.h + static_cast<size_t>(col) * ep.F + fg) = *src;
         }
-        if (!ALT) named_bar(1, kEpiThreads);
+        if (!WIDE) named_bar(1, kEpiThreads);
     }
     if constexpr (EPI == EPI_RESID && PASS == 1) {
         // the staged chunk: thread t stores token t/8, features 16 (t%8) .. +15 of the tile
@@ -492,18 +475,9 @@ __device__ __forceinline__ void epilogue_c32(const EpiArgs& ep, const GemmPlan& 
 #pragma unroll
             for (int i = 0; i < 2; ++i) dst[i] = src[i];
         }
-        if (!ALT) named_bar(1, kEpiThreads);  // the staging memory is free again
+        if (!WIDE) named_bar(1, kEpiThreads);  // the staging memory is free again
     }
-    if constexpr (EPI == EPI_RESID && PASS == 0) {
-        named_bar(1, kEpiThreads);
-        if (e < 32) {
-            const int col = col0 + lane;
-            const float* rd = sm.red + (c_in / 32) * 128;
-            if (col < p.N)
-                ep.sq_out[static_cast<size_t>(mt) * p.N + col] = ((rd[lane] + rd[32 + lane]) + rd[64 + lane]) + rd[96 + lane];
-        }
-        named_bar(1, kEpiThreads);
-    } else if constexpr (EPI == EPI_RESID && PASS == 2) {
+    if constexpr (EPI == EPI_RESID && PASS == 2) {
         // the chunk's four quarter sums, written by its first pass (the barriers since then order
         // them; the next writer of these words comes after the tile's next barrier)
         if (e < 32) {
@@ -676,11 +650,9 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
     const int nchunks = p.ntile / 32;
     constexpr int kPass1 = EPI == EPI_RESID ? 1 : 0;  // the residual epilogue runs in two passes
     const size_t slot_floats = static_cast<size_t>(p.ntile) * kBM;
-    // TMEM: two accumulators of acc_cols columns, then (token tiles up to 128) the staged old
-    // residual of the finisher's tile, x_cols columns
-    const uint32_t t_x =
-        !WIDE && ca.x_cols ? tmem_base + static_cast<uint32_t>(ca.x_col0) + (static_cast<uint32_t>(quarter * 32) << 16)
-                  : 0u;
+    // TMEM: the accumulators, then (32-token tiles) the staged old residual of the finisher's
+    // tile, x_cols columns from x_col0
+    const uint32_t t_x = tmem_base + static_cast<uint32_t>(ca.x_col0) + (static_cast<uint32_t>(quarter * 32) << 16);
     int rs_nt = -1, ids_nt = -1;
     int prepared = -1;
     float v[16];
@@ -709,18 +681,14 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
                 ids_nt = pnt;
             }
         }
-        if constexpr (EPI == EPI_RESID) {
-            if (t_x) {
-                const int row = pmt * kBM + rt;
-                for (int c = 0; c < nchunks; ++c) {
+        if constexpr (EPI == EPI_RESID && !WIDE) {
+            const int row = pmt * kBM + rt;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int col = pnt * p.ntile + c * 32 + half * 16 + j;
-                        v[j] = (row < p.M && col < p.N) ? ep.out[static_cast<size_t>(col) * ep.ld_out + row] : 0.0f;
-                    }
-                    tmem_st_32x16(t_x + static_cast<uint32_t>(c * 32 + half * 16), v);
-                }
+            for (int j = 0; j < 16; ++j) {
+                const int col = pnt * p.ntile + half * 16 + j;
+                v[j] = (row < p.M && col < p.N) ? ep.out[static_cast<size_t>(col) * ep.ld_out + row] : 0.0f;
             }
+            tmem_st_32x16(t_x + static_cast<uint32_t>(half * 16), v);
         }
     };
     // Wide tiles read the old residual from global memory (TMEM has no room to stage it; a warp's
@@ -798,9 +766,8 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
                     if (c + 1 < nchunks) load_x(mt, nt, c + 1);
                 }
                 epilogue_c32<EPI, kPass1, WIDE>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
-                                                t_acc + static_cast<uint32_t>(c * 32),
-                                                t_x ? t_x + static_cast<uint32_t>(c * 32) : 0u, esm, e, half, quarter,
-                                                lane, status, x_ahead || !WIDE ? v : nullptr, nullptr, x_ahead, es.buf);
+                                                t_acc + static_cast<uint32_t>(c * 32), t_x, esm, e, half, quarter,
+                                                lane, status, x_ahead || !WIDE ? v : nullptr, nullptr, es.buf);
                 es.buf ^= 1;
             }
         }
@@ -963,8 +930,8 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
                         if (c + n_own < nchunks) load_x(mt, nt, c + n_own);
                     }
                     epilogue_c32<EPI, kPass1, true>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
-                                              t_acc + static_cast<uint32_t>(c * 32), 0u, esm, e, half, quarter, lane,
-                                              status, v, nullptr, EPI == EPI_RESID, es.buf);
+                                              t_acc + static_cast<uint32_t>(c * 32), t_x, esm, e, half, quarter, lane,
+                                              status, v, nullptr, es.buf);
                     es.buf ^= 1;
                 }
             }
@@ -997,7 +964,7 @@ __device__ __forceinline__ void chain_phase_epilogue(const ChainArgs& ca, int ph
 #pragma unroll 1
                 for (int c = WIDE && reducer ? part : 0; c < nchunks; c += WIDE && reducer ? n_own : 1)
                     epilogue_c32<EPI, 2>(ep, p, mt, nt * p.ntile + c * 32, c * 32, rt,
-                                         t_acc + static_cast<uint32_t>(c * 32), 0u, esm, e, half, quarter,
+                                         t_acc + static_cast<uint32_t>(c * 32), t_x, esm, e, half, quarter,
                                          lane, status);
                 if (P.done2 || (WIDE && reducer)) {
                     named_bar(1, kEpiThreads);
