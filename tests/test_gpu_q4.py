@@ -44,8 +44,8 @@ def test_q4_weights_dequantise_to_the_oracles(pkg):
 
 @pytest.mark.parametrize("n_prompt", [64, 192])
 def test_q4_blockwise_teacher_forced(pkg, n_prompt):
-    """The 4-bit block loop against the oracle; a 192-token prompt puts the prefill on token
-    tiles too wide for tensor-memory A stages (the shared-memory stages and their own rings)."""
+    """The 4-bit block loop against the oracle, prefill of 64 and of 192 tokens (a model this small
+    runs whole 32-token tiles, its A stages in shared memory; wider tiles: test_gpu_wide.py)."""
     from test_gpu_step import _run_teacher_forced
     model = O.Model(O.OracleConfig(weight_bits=4))
     prompt = I.uniform_prompt(n_prompt, 1024, 1023, seed=31)

@@ -1,8 +1,10 @@
 """Split tiles of wide token tiles, and query tiles cut from a K/V head's whole group, at the sizes
-where their bookkeeping can go wrong, against the same sums in 64 bits."""
+where their bookkeeping can go wrong, against the same sums in 64 bits; and windows of such tiles
+through whole layers, with bf16 weights against the oracle, with 4-bit ones against 64 bits."""
 import numpy as np
 import pytest
 
+import dllm_inputs as I
 import oracle as O
 
 torch = pytest.importorskip("torch")
@@ -42,19 +44,34 @@ def test_wide_split_tiles(pkg, M, N, K, grid):
     assert torch.equal(D, pkg.dllm_op_gemm(W, X, M, N, K, grid=grid))
 
 
-# the last sizes whose tiles run whole, 32 tokens and one CTA each (up to 960 columns deep, at most
-# one tile per SM), and the first past them
-@pytest.mark.parametrize("M,N,K", [
-    (768, 33, 256), (128, 1, 8), (2432, 256, 960), (2433, 256, 960), (2432, 250, 968), (256, 2432, 688),
-    (256, 2433, 688), (128, 4096, 64), (130, 31, 960), (130, 31, 968),
+# Sizes (for s SMs) whose tiles run whole, 32 tokens and one CTA each: up to 15 k-blocks of 64 and at
+# most one tile per SM, eight token tiles counted for up to 256 tokens; the last ones and the first
+# past them.  small: which it is, seen by the number of CTAs.
+@pytest.mark.parametrize("small,size", [
+    (True, lambda s: (768, 33, 256)), (True, lambda s: (128, 1, 8)),
+    (True, lambda s: (128 * (s // 8), 256, 960)), (False, lambda s: (128 * (s // 8) + 1, 256, 960)),
+    (True, lambda s: (128 * (s // 8 - 1), 250, 960)), (False, lambda s: (128 * (s // 8 - 1), 250, 968)),
+    (True, lambda s: (256, 32 * (s // 2), 688)), (False, lambda s: (256, 32 * (s // 2) + 1, 688)),
+    (True, lambda s: (128, 32 * (s - 1), 64)), (True, lambda s: (130, 31, 960)), (False, lambda s: (130, 31, 968)),
 ])
-def test_small_whole_tiles(pkg, M, N, K):
+def test_small_whole_tiles(pkg, small, size):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    M, N, K = size(sms)
     g = torch.Generator().manual_seed(M + N + K)
     W, X = _bf16(g, M, K, sigma=0.05), _bf16(g, N, K)
     D = pkg.dllm_op_gemm(W, X, M, N, K)
     w, x = W.double(), X.double()
     tol = 1e-5 * x.norm(dim=1)[:, None] * w.norm(dim=1)[None, :]  # as above
     assert bool(((D.double() - x @ w.T).abs() <= tol).all())
+    mt, kb = (M + 127) // 128, (K + 63) // 64
+    _, trace = pkg.dllm.dllm_op_gemm_trace(W, X, M, N, K, 1)
+    assert (len(trace) == mt * ((N + 31) // 32)) == small
+    if small:  # the sums are those of 32 rows alone, and of one k-block per CTA, bit for bit
+        n = min(N, 32)
+        first = pkg.dllm_op_gemm(W, X[:n].contiguous(), M, n, K)
+        assert torch.equal(D[:n], first)
+        if mt * kb < sms:
+            assert torch.equal(first, pkg.dllm_op_gemm(W, X[:n].contiguous(), M, n, K, grid=mt * kb))
 
 
 @pytest.mark.parametrize("V,N,d", [(1024, 251, 4096), (512, 96, 2048), (4096, 64, 512)])
@@ -119,18 +136,135 @@ def test_head_argmax_ties(pkg, N):
         assert abs(float(conf[n]) - p) <= 1e-5 * p  # a sum of at most 384 exponentials in fp32
 
 
-# 4-bit weights: the expanded tiles in tensor memory with 5 and 4 stages, then in shared memory
+# One layer of LLaDA-8B's width under a small vocabulary
+SHAPE = dict(n_layers=1, d_model=4096, n_heads=32, head_dim=128, ffn=12288, vocab=1024, mask_id=1023,
+             rope_base=500000.0)
+
+
+def _weights(ctx):
+    """The context's embedding, projections and head in 64 bits."""
+    w = {i: ctx.dllm_get_weight(0, i) for i in range(7)} | {"emb": ctx.dllm_get_weight(-1, 1), "head": ctx.dllm_get_weight(-1, 2)}
+    return {k: torch.from_numpy(v.view(np.int16)).cuda().view(torch.bfloat16).double() for k, v in w.items()}
+
+
+def _one_layer(w, tok, pk, pv, r=lambda t: t):
+    """Logits of the window `tok` after the prefix keys and values pk, pv [P][H][hd] through one layer and the
+    head, in 64 bits; r is applied where the kernels round to bf16."""
+    H, hd, T, P = SHAPE["n_heads"], SHAPE["head_dim"], len(tok), pk.shape[0]
+    ang = torch.arange(P, P + T, device="cuda").double()[:, None] * SHAPE["rope_base"] ** (
+        -torch.arange(0, hd, 2, device="cuda").double() / hd)[None, :]
+    cs, sn = ang.cos()[:, None], ang.sin()[:, None]
+
+    def rms(x):
+        return (x.square().mean(-1, keepdim=True) + 1e-5).rsqrt()
+
+    def rope(x):
+        a, b = x[..., :hd // 2], x[..., hd // 2:]
+        return torch.cat([a * cs - b * sn, b * cs + a * sn], -1)
+
+    x = w["emb"][tok]
+    q, k, v = ((x @ w[i].T * rms(x)).view(T, H, hd) for i in range(3))
+    q, k, v = r(rope(q)), torch.cat([pk, r(rope(k))]), torch.cat([pv, r(v)])
+    p = torch.softmax(torch.einsum("thd,nhd->htn", q, k) / hd ** 0.5, -1)
+    x = x + r(torch.einsum("htn,nhd->thd", r(p), v).reshape(T, H * hd)) @ w[3].T
+    g, u = (r(x) @ w[i].T * rms(x) for i in (4, 5))
+    x = x + r(torch.nn.functional.silu(g) * u) @ w[6].T
+    return r(x) @ w["head"].T * rms(x)
+
+
+@pytest.fixture(scope="module")
+def q4_weights(pkg):
+    ctx = pkg.Context(pkg.Config(weight_bits=4, **SHAPE))
+    yield _weights(ctx)
+    ctx.close()
+
+
+# 4-bit weights: the expanded tiles in tensor memory with 6 and 4 stages, then in shared memory; last
+# chunks of one token and whole ones
 @pytest.mark.parametrize("T", [33, 64, 65, 128, 129])
-def test_q4_wide_windows(pkg, T):
-    from perf import cases
-    case = dict(name="", kind="step", shape="llada", layers=1, B=1, P=70, T=T, masked=T // 2, bits=4, cache=True,
-                vocab=1024)
-    got = torch.as_tensor(cases.run(cases.prepare(case, 7))["logits"]).double().cuda()
-    ref = cases.exact(case, 7)["logits"]
-    assert got.shape == ref.shape
-    # A layer and the head round to bf16 (2^-9) eight times in a row (embedding, q/k/v, probabilities,
-    # attention output, x, h, x; the weights are exact): sqrt(8) 2^-9 = 5.5e-3 where the errors' signs
-    # are random.  By the median row: the 4-bit draws' mean is not zero, so a row's state lies along
-    # one direction with the sign of a sum, and a row whose sum is close to 0 amplifies any rounding.
-    err = ((got - ref).norm(dim=-1) / ref.norm(dim=-1)).flatten()
-    assert err.median() <= 5.5e-3
+def test_q4_wide_windows(pkg, q4_weights, T):
+    P = 70
+    ctx = pkg.Context(pkg.Config(weight_bits=4, max_ctx=P + T, max_window=T, block_len=T, **SHAPE))
+    ctx.dllm_set_prefix_kv_random(pkg.Sched(), 1, P, T, 7)
+    ctx.dllm_begin_block()
+    tok = I.uniform_prompt(P + T, 1024, 1023, seed=T)[None]
+    st = np.full((1, P + T), pkg.COMMITTED, np.uint8)
+    st[0, :P] = pkg.FIXED
+    tok[0, P + T // 2], st[0, P + T // 2] = 1023, pkg.MASKED
+    ctx.dllm_set_state(tok, st)
+    ctx.dllm_set_debug(1)
+    ctx.dllm_denoise_step()
+    got = torch.as_tensor(ctx.dllm_get_step_debug(logits=True)["logits"][0]).double().cuda()
+    pk, pv = (torch.as_tensor(ctx.dllm_get_kv(0, i, 0, 0, P)).double().cuda().view(P, 32, 128) for i in (0, 1))
+    ctx.close()
+    win = torch.as_tensor(tok[0, P:]).long().cuda()
+    ref = _one_layer(q4_weights, win, pk, pv)
+
+    # Every row within 5 times what bf16 roundings do to it: the largest of 16 draws of errors of
+    # random sign and up to bf16's largest relative size, 2^-9, at every place where the kernels
+    # round.  The 4-bit draws' mean is not zero, so a row's state lies along one direction with the
+    # sign of a sum, and in a row whose sum is close to 0 any rounding grows (to 30 %); the others,
+    # a last chunk's last row among them, must stay within a thousandth or so.
+    def off(z):
+        return (z - ref).norm(dim=-1) / ref.norm(dim=-1)
+
+    gen = torch.Generator(device="cuda").manual_seed(T)
+
+    def rounding(t):
+        return t * (1 + 2.0 ** -9 * (2 * torch.rand(t.shape, device="cuda", dtype=torch.float64, generator=gen) - 1))
+
+    spread = torch.stack([off(_one_layer(q4_weights, win, pk, pv, rounding)) for _ in range(16)]).amax(0)
+    assert bool((off(got) <= 5 * spread).all())
+    assert float(spread.median()) <= 1e-3 and float(spread[-1]) <= 1e-2
+
+
+# Windows and lookahead windows of several 32-token chunks through two layers of LLaDA-8B's width,
+# without and with refresh rows (chunks of window rows, of refresh rows and of both): block length,
+# prompt, tokens to generate, schedule
+@pytest.fixture(scope="module")
+def wide_model():
+    return O.Model(O.OracleConfig(**(SHAPE | {"n_layers": 2})))
+
+
+@pytest.mark.parametrize("block,P,gen,kw", [
+    (33, 70, 33, {}), (129, 20, 129, {}), (251, 12, 251, {}),
+    (32, 70, 96, dict(spec_blocks=2, spec_trigger=32)),
+    (33, 40, 66, dict(scr_rows=8, theta_stable=2.0)), (96, 40, 192, dict(scr_rows=32, theta_stable=2.0)),
+])
+def test_wide_windows_teacher_forced(pkg, wide_model, block, P, gen, kw):
+    from test_gpu_step import _run_teacher_forced
+    kw = dict(steps_per_block=1, **kw)
+    # n bf16 roundings of random sign, 2^-9 / sqrt(3) of a value each: three times what they sum to.
+    # A layer has eight (q, k, v, probabilities, attention output, x, h, x), keys and values one more.
+    def bound(n):
+        return 3 * (n / 3) ** 0.5 * 2.0 ** -9
+
+    def rows_off(a, b):
+        return float((np.linalg.norm(a - b, axis=-1) / np.linalg.norm(b, axis=-1)).max())
+
+    seen = {"T": set(), "rows": 0}
+
+    def check(sess, ctx, oo, go, before, o_after, g_after):
+        got, ref = ctx.dllm_get_step_debug(logits=True)["logits"][0], sess.decisions(logits=True)["logits"]
+        assert rows_off(got, ref) <= bound(16)
+        seen["T"].add(sess.window()["T"])
+        if kw.get("scr_rows"):
+            od, gd = sess.scr_decisions(), ctx.dllm_get_scr_debug()
+            n = len(od["pos"])
+            assert np.array_equal(gd["pos"][:n], od["pos"]) and (gd["pos"][n:] == -1).all()
+            assert np.allclose(gd["conf"][:n], od["conf"], rtol=0.05)
+            assert np.allclose(gd["tokconf"][:n], od["tokconf"], rtol=0.05)
+            assert go["n_refreshed"] == oo["n_refreshed"]
+            seen["rows"] += n
+        for layer in (0, 1):  # every cached row, refreshed ones included
+            for which in (0, 1):
+                ref = sess.prefix_kv(layer, which)
+                got = ctx.dllm_get_kv(layer, which, 0, 0, ref.shape[0])
+                assert rows_off(got, ref) <= bound(8 * layer + 1)
+
+    ctx = pkg.Context(pkg.Config(max_ctx=P + gen, max_window=max(P, 3 * block if "spec_blocks" in kw else block + 32),
+                                 block_len=block, **(SHAPE | {"n_layers": 2})))
+    _run_teacher_forced(wide_model, O.OracleSched(block_len=block, **kw), pkg.Sched(**kw),
+                        I.uniform_prompt(P, 1024, 1023, seed=block), gen, ctx, check)
+    ctx.close()
+    assert max(seen["T"]) == (96 if block == 32 else block) and (seen["rows"] > 0) == ("scr_rows" in kw)
