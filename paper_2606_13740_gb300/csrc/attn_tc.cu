@@ -132,7 +132,7 @@ template <int NB>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_attn_tc(const __grid_constant__ TcMaps maps, const int* __restrict__ seq_kv, __nv_bfloat16* __restrict__ out,
               int T, int H, int Hkv, int cap, int qtiles, int csize, int qx, int* status,
-              unsigned long long* trace) {
+              unsigned long long* trace, int z0) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* sQ = smem;                       // 32 KB
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     pdl_launch_dependents();
     // hk: the K/V head; its H / Hkv query heads' rows, head by head, are one run of q
     const int split = blockIdx.x, hk = blockIdx.y, nrows = H / Hkv * T;
-    const int b = blockIdx.z / qtiles, qt = blockIdx.z - b * qtiles;
+    const int bt = z0 + static_cast<int>(blockIdx.z), b = bt / qtiles, qt = bt - b * qtiles;
     const int NK = seq_kv[b] + T - qx;  // the last qx rows are queries only
     const int nblk = (NK + kTcKeys - 1) / kTcKeys;
     const int blk0 = split * nblk / csize, blk1 = (split + 1) * nblk / csize;
@@ -539,12 +539,22 @@ size_t tc_smem() {
 }
 
 template <int NB>
-cudaError_t tc_go(cudaLaunchConfig_t& cfg, const TcMaps& maps, const int* seq_kv, __nv_bfloat16* out, int T, int H,
-                  int Hkv, int cap, const AttnPlan& a, int* status, unsigned long long* trace) {
+cudaError_t tc_go(cudaLaunchConfig_t& cfg, const TcMaps& maps, const int* seq_kv, __nv_bfloat16* out, int B, int T,
+                  int H, int Hkv, int cap, const AttnPlan& a, int* status, unsigned long long* trace) {
     cfg.blockDim = dim3(kTcThreads);
     cfg.dynamicSmemBytes = tc_smem<NB>();
-    return cudaLaunchKernelEx(&cfg, k_attn_tc<NB>, maps, seq_kv, out, T, H, Hkv, cap, a.qtiles, a.csize, a.qx, status,
-                              trace);
+    // A launch takes 65535 query tiles of all sequences; a group's many (256 of 1024 tokens under 32
+    // query heads) pass that at 256 sequences.  (As one dimension of clusters the divisions cost every
+    // CTA its start: 12 x 17 tokens of 32 heads over 4000 keys 114 -> 117 us.)
+    constexpr long long kMaxZ = 65535;
+    const long long tiles = static_cast<long long>(B) * a.qtiles;
+    cudaError_t e = cudaSuccess;
+    for (long long z0 = 0; z0 < tiles && e == cudaSuccess; z0 += kMaxZ) {
+        cfg.gridDim = dim3(a.csize, Hkv, static_cast<unsigned>(tiles - z0 < kMaxZ ? tiles - z0 : kMaxZ));
+        e = cudaLaunchKernelEx(&cfg, k_attn_tc<NB>, maps, seq_kv, out, T, H, Hkv, cap, a.qtiles, a.csize, a.qx, status,
+                               trace, static_cast<int>(z0));
+    }
+    return e;
 }
 
 }  // namespace
@@ -599,7 +609,6 @@ cudaError_t launch_attention_tc(const __nv_bfloat16* q, const __nv_bfloat16* kc,
         !make_tmap_bf16(&maps.v, vc, static_cast<uint64_t>(B) * Hkv * cap, 128, kTcKeys))
         return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(a.csize, Hkv, B * a.qtiles);
     cfg.stream = st;
     cudaLaunchAttribute at[2];
     int n = 0;
@@ -615,8 +624,8 @@ cudaError_t launch_attention_tc(const __nv_bfloat16* q, const __nv_bfloat16* kc,
     }
     cfg.attrs = at;
     cfg.numAttrs = n;
-    return a.nb == 2 ? tc_go<2>(cfg, maps, seq_kv, out, T, H, Hkv, cap, a, status, trace)
-                     : tc_go<1>(cfg, maps, seq_kv, out, T, H, Hkv, cap, a, status, trace);
+    return a.nb == 2 ? tc_go<2>(cfg, maps, seq_kv, out, B, T, H, Hkv, cap, a, status, trace)
+                     : tc_go<1>(cfg, maps, seq_kv, out, B, T, H, Hkv, cap, a, status, trace);
 }
 
 }  // namespace dllm

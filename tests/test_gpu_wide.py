@@ -112,6 +112,20 @@ def test_group_query_tiles(pkg, B, T, H, Hkv, kv):
         assert (got - ref).abs().max() <= 0.05 * ref.abs().max()
 
 
+def test_group_query_tiles_past_65535(pkg):
+    """256 sequences of 256 query tiles each (one K/V head, 32 query heads, 1024 tokens): the first and
+    the last sequence."""
+    B, T, H = 256, 1024, 32
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q, k, v = (torch.randn(*s, device="cuda", generator=g, dtype=torch.bfloat16)
+               for s in ((B, H, T, 128), (B, 1, T, 128), (B, 1, T, 128)))
+    out = pkg.dllm_op_attention(q, k, v, torch.zeros(B, dtype=torch.int32).cuda(), B, T, H, 128, T, 0, Hkv=1)
+    for b in (0, B - 1):
+        ref = torch.softmax(q[b].double() @ k[b].double().transpose(1, 2) / 128 ** 0.5, -1) @ v[b].double()
+        got = out.view(B, T, H, 128)[b].transpose(0, 1).double()
+        assert (got - ref).norm() <= 1e-2 * ref.norm()  # bf16 probabilities and outputs
+
+
 @pytest.mark.parametrize("N", [32, 40])
 def test_head_argmax_ties(pkg, N):
     """Equal largest logits in one warp's rows, in two quarters, in two tiles and beside the mask id:
