@@ -28,9 +28,9 @@
 // the tile's parts but the last: one finisher took the columns one after
 // another, and with five parts and 256 tokens (the output projection of a
 // 251-token window) that was 40 slices in a row on a sixth of the SMs (a layer
-// at 251 tokens 190 -> 132 us, at 160 tokens and ffn 18944 163 -> 104 us).  Every CTA waits only on CTAs
-// that wait on nothing later than it, and the grid never exceeds the SM count,
-// so all are resident.
+// at 251 tokens 190 -> 132 us, at 160 tokens and ffn 18944 163 -> 104 us).  Every CTA publishes its
+// part of a tile before it waits for others', in the order of its range, and
+// the grid never exceeds the SM count, so all are resident.
 // The weights (the context's, stored tile-major) arrive as one contiguous
 // bulk copy per 16 KB tile; row-major weights of the single-projection entry
 // points arrive through a 2-D tensor map.

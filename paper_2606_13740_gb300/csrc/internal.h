@@ -166,8 +166,8 @@ struct ChainMaps {
     CUtensorMap w[kMaxPhases];
     CUtensorMap x[kMaxPhases];
 };
-// Fills grid, stages, ntile, acc_cols, x_cols, tmem_cols and smem from the phases' plans for a shared-memory budget (bytes, <= 227 KB).  False if the
-// phases do not share one token tiling.
+// Fills grid, stages, ntile, acc_cols, x_cols, tmem_cols and smem from the phases' plans for a
+// shared-memory budget (bytes, <= 227 KB).  False if the phases do not share one token tiling.
 bool chain_plan(ChainArgs& ca, int smem_budget);
 constexpr int kChainSmemFull = 227 * 1024;    // one CTA per SM, deepest ring
 constexpr int kChainSmemShared = 146 * 1024;  // leaves room for two attention CTAs beside it
